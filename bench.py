@@ -391,9 +391,9 @@ def main():
             cc_line = {"bound": "alu", "kernel": kname + " (FP32 contraction + inverse angular DFT + argmax)",
                        "achieved": flops / cc_s / 1e12, "peak": alu_peak, "unit": "TFLOP/s", "peak_source": alu_src}
         else:
-            kname = {256: "cc_tc256_kernel", 512: "cc_tc512_kernel"}.get(info["M"], "cc_tc_kernel")
-            if info["M"] == 256 and choice["kernel"] == mra.MRA_KERNEL_TCGEN05:
-                kname = "cc_umma256_kernel"
+            kname = {256: "cc_hybrid256_kernel", 512: "cc_tc512_kernel"}.get(info["M"], "cc_tc_kernel")
+            if info["M"] == 256 and choice["kernel"] == mra.MRA_KERNEL_MMA_SYNC:
+                kname = "cc_tc256_kernel"
             tc_idft = info["M"] in (256, 512)  # the inverse DFT on tensor cores too (M <= 128: FP32)
             flops = pairs_per_launch * (f_con + (f_ifft if tc_idft else 0))
             cc_line = {"bound": "tensor", "kernel": kname + " (16-bit tensor-core contraction"
@@ -462,7 +462,7 @@ def main():
     if not args.no_compare and prec != mra.MRA_FP32:
         cmp_res = run_path(mra.MRA_FP32, "fp32", w, refs, imgs, n, args.steps, args.warmup)
         cmp_res["al"].close()
-    # the same 16-bit step on the tcgen05 contraction kernel (M = 256 only), its own roofline
+    # the same 16-bit step on the kernel with the tcgen05 inverse DFT (M = 256 only), its own roofline
     umma_res = None
     if (not args.no_compare and prec != mra.MRA_FP32 and world == 1 and
             max(nr for _, nr in ring_table(w.first_ring, w.last_ring, w.ring_step)) == 256):
@@ -557,9 +557,8 @@ def main():
                                     "roofline": umma_res["roofline"], "stages": umma_res["prof"],
                                     "gpu_launches": umma_res["gpu_launches"], "launch": umma_res["launch"],
                                     "clocks": umma_res["clocks"],
-                                    "note": "the headline step with the tcgen05 / TMEM contraction kernel "
-                                            "(MRA_KERNEL_TCGEN05) at the library's default chunk; the autotuner "
-                                            "keeps mma.sync for the headline where it is faster"}
+                                    "note": "the headline step with the tcgen05 / TMEM kernel "
+                                            "(MRA_KERNEL_TCGEN05) at the library's default chunk"}
         print(json.dumps(line), flush=True)
     al.close()
     if world > 1:

@@ -73,10 +73,11 @@ enum mra_precision {
  * two compute the same table and differ only in speed.  Other M and the
  * FP32 path ignore the choice. */
 enum mra_kernel {
-    MRA_KERNEL_AUTO = 0,     /* the library's default (MRA_KERNEL_MMA_SYNC)                    */
-    MRA_KERNEL_MMA_SYNC = 1, /* warp-level mma.sync, tiles of 8 rows x 8 references            */
-    MRA_KERNEL_TCGEN05 = 2   /* tcgen05.mma with TMEM accumulators and TMA tensor-map staging,
-                                tiles of 16 rows x 8 references (k_umma256.cu)                  */
+    MRA_KERNEL_AUTO = 0,     /* the library's default (the kernel of MRA_KERNEL_TCGEN05)       */
+    MRA_KERNEL_MMA_SYNC = 1, /* warp-level mma.sync throughout                                 */
+    MRA_KERNEL_TCGEN05 = 2   /* mma.sync contraction, tcgen05.mma inverse angular DFT with the
+                                angular sums accumulated in TMEM (k_umma256.cu); boxes of about
+                                L = 200 that only fit MRA_KERNEL_MMA_SYNC's layout run that       */
 };
 
 /* Search configuration.  Validated by mra_create:

@@ -3,9 +3,8 @@
 The library exposes two launch choices per handle (``mra_config_t``):
 
 * ``kernel``: for the 16-bit paths at M = 256, the warp-level mma.sync
-  kernel (tiles of 8 rows x 8 references, two CTAs per SM) or the tcgen05
-  kernel (tiles of 16 rows x 8 references, TMEM accumulators, one persistent
-  CTA per SM);
+  kernel (two CTAs per SM) or the kernel with the tcgen05 inverse DFT (TMEM
+  accumulators, one persistent CTA per SM; also the library's own choice);
 * ``chunk_images``: images per internal chunk (the particle spectra of one
   chunk are the largest workspace; fewer, larger chunks mean fewer launches
   and kernel tails, smaller ones a smaller footprint).  Candidates: the

@@ -13,11 +13,11 @@
 // (p rows) for 8 rows x 4 references.  A tile of 8 rows x 8 references is
 // two such MMAs per k-step.  Operands are BF16 (or FP16), accumulation FP32.
 //
-// For M = 256 (rings up to 40) the per-pair angular state is kept as BF16 in
-// shared memory and the inverse angular DFT runs on tensor cores too
-// (cc_tc256_kernel); for M = 512 the state is BF16 and the inverse DFT runs
-// in FP32 (cc_tc512_kernel); for M <= 128 the state stays FP32
-// (cc_tc_kernel).  Either way the row maxima select the 8 rows
+// For M = 256 (rings up to 40) and M = 512 the per-pair angular state is kept
+// as BF16 in shared memory and the inverse angular DFT runs on tensor cores
+// too (cc_tc256_kernel, cc_tc512_kernel); for M <= 128 the state stays FP32
+// (cc_tc_kernel).  (The default at M = 256 is the kernel of k_umma256.cu;
+// cc_tc256_kernel serves MRA_KERNEL_MMA_SYNC.)  Either way the row maxima select the 8 rows
 // (reference, shift, mirror) per image that the rescore kernel recomputes
 // from scratch in FP32; its argmax is the answer.
 #include <cuda_bf16.h>
@@ -41,28 +41,29 @@ __device__ __forceinline__ uint32_t pack16x2(uint16_t lo, uint16_t hi) {
 }
 
 // ---------------------------------------------------------------------------
-// Reference B fragments: [ref tile of 8][N-block 2][KS][lane 32] x uint2.
-// Lane 4g + t of N-block nb holds column g = (reference 4 nb + g/2, value
-// v if g even else u) at k = 2t, 2t+1 (first word) and 2t+8, 2t+9 (second).
+// Reference B fragments: [ref tile of 8][KS][lane 32] x uint4, the two words
+// of both N-blocks of 4 references side by side, so that a lane fetches a
+// k-step with one 16-byte load.  Lane 4g + t of N-block nb holds column g =
+// (reference 4 nb + g/2, value v if g even else u) at k = 2t, 2t+1 (first
+// word) and 2t+8, 2t+9 (second).
 // ---------------------------------------------------------------------------
-__global__ void refs16_kernel(Geometry g, const float2 *__restrict__ B, int ktiles, uint2 *B16, bool fp16) {
-  const int64_t total = static_cast<int64_t>(ktiles) * g.KS * 64;
+__global__ void refs16_kernel(Geometry g, const float2 *__restrict__ B, int ktiles, uint4 *B16, bool fp16) {
+  const int64_t total = static_cast<int64_t>(ktiles) * g.KS * 32;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
        idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int lane = static_cast<int>(idx & 31);
     const int64_t r = idx >> 5;
     const int kk = static_cast<int>(r % g.KS);
-    const int nb = static_cast<int>((r / g.KS) & 1);
-    const int kt = static_cast<int>(r / g.KS / 2);
+    const int kt = static_cast<int>(r / g.KS);
     const int2 ki = g.ksinfo[kk];
     const int2 seg = g.fseg[ki.x];
     const int gi = lane >> 2, t = lane & 3;
-    const int refl = 4 * nb + (gi >> 1), c = gi & 1;
+    const int c = gi & 1;
     const int ks[4] = {2 * t, 2 * t + 1, 2 * t + 8, 2 * t + 9};
-    uint16_t v[4];
+    uint16_t v[8];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int rr = 16 * ki.y + ks[e];
+    for (int e = 0; e < 8; ++e) {
+      const int rr = 16 * ki.y + ks[e & 3], refl = 4 * (e >> 2) + (gi >> 1);
       float val = 0.f;
       if (rr < seg.y) {
         const float2 X = B[(static_cast<int64_t>(kt) * g.NB + seg.x + rr) * kTile + refl];
@@ -70,7 +71,7 @@ __global__ void refs16_kernel(Geometry g, const float2 *__restrict__ B, int ktil
       }
       v[e] = to16(val, fp16);
     }
-    B16[idx] = make_uint2(pack16x2(v[0], v[1]), pack16x2(v[2], v[3]));
+    B16[idx] = make_uint4(pack16x2(v[0], v[1]), pack16x2(v[2], v[3]), pack16x2(v[4], v[5]), pack16x2(v[6], v[7]));
   }
 }
 
@@ -95,14 +96,15 @@ template <int M, int KT_>
 struct TcShape {
   static constexpr int RT = kTile, KT = KT_, PAIRS = RT * KT;
   static constexpr int NBLK = KT / 4;  // MMAs (N-blocks of 4 references) per k-step
+  static_assert(KT == kTile, "a k-step's B fragment holds the tile's two N-blocks");
   static constexpr int WARPS = 16, THREADS = 32 * WARPS;
   static constexpr int P = IfftShape<M>::P;  // float2 per pair buffer
   static constexpr size_t STATE = static_cast<size_t>(PAIRS) * P * sizeof(float2);
   static constexpr size_t TW = M * sizeof(float2);
   static constexpr size_t BARS = WARPS * sizeof(uint64_t);
-  // A: ks_max k-steps x 512 B, then B: NBLK x ks_max x 256 B
+  // A: ks_max k-steps x 512 B, then B the same
   __host__ __device__ static size_t stage_bytes(int ks_max) {
-    return static_cast<size_t>(ks_max) * 512 + static_cast<size_t>(NBLK) * ks_max * 256;
+    return static_cast<size_t>(ks_max) * 1024;
   }
   __host__ __device__ static size_t smem(int ks_max) { return STATE + TW + BARS + WARPS * stage_bytes(ks_max); }
 };
@@ -334,9 +336,7 @@ __global__ void __launch_bounds__(kTc256Threads, 2) cc_tc256_kernel(Geometry g, 
     fence_proxy_async();
     mbar_arrive_expect_tx(full + (q & 1), nks * 1024u);
     bulk_g2s(dst, a.A16 + (rt * g.KS + k0) * 32, nks * 512u, full + (q & 1));
-    bulk_g2s(dst + nks * 512u, a.B16 + ((static_cast<int64_t>(kt) * 2) * g.KS + k0) * 32, nks * 256u, full + (q & 1));
-    bulk_g2s(dst + nks * 768u, a.B16 + ((static_cast<int64_t>(kt) * 2 + 1) * g.KS + k0) * 32, nks * 256u,
-             full + (q & 1));
+    bulk_g2s(dst + nks * 512u, a.B16 + (static_cast<int64_t>(kt) * g.KS + k0) * 32, nks * 512u, full + (q & 1));
   };
   if (tid == 0) {
     issue(0);
@@ -381,8 +381,7 @@ __global__ void __launch_bounds__(kTc256Threads, 2) cc_tc256_kernel(Geometry g, 
         const int kbase = s_kso[f0];
         const int nks_c = s_kso[f1] - kbase;
         const uint4 *stA = reinterpret_cast<const uint4 *>(stage + buf * kTc256Stage) + lane;
-        const uint2 *stB0 = reinterpret_cast<const uint2 *>(stage + buf * kTc256Stage + static_cast<size_t>(nks_c) * 512) + lane;
-        const uint2 *stB1 = stB0 + nks_c * 32;
+        const uint4 *stB = stA + nks_c * 32;
         for (int f = f0 + warp; f < f1; f += kTc256Warps) {
           const int jb = s_kso[f] - kbase, nj = s_kso[f + 1] - s_kso[f];  // 1..3 k-steps
           float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -390,9 +389,9 @@ __global__ void __launch_bounds__(kTc256Threads, 2) cc_tc256_kernel(Geometry g, 
           for (int jj = 0; jj < 3; ++jj) {
             if (jj < nj) {
               const int j = (jb + jj) * 32;
-              const uint4 af = stA[j];
-              mma16816<FP16>(d0, af, stB0[j]);
-              mma16816<FP16>(d1, af, stB1[j]);
+              const uint4 af = stA[j], bf = stB[j];
+              mma16816<FP16>(d0, af, make_uint2(bf.x, bf.y));
+              mma16816<FP16>(d1, af, make_uint2(bf.z, bf.w));
             }
           }
           // lane (g8, t4): d[0..1] = Re/Im Z(f), d[2..3] = Im/Re Z(M - f)
@@ -514,9 +513,7 @@ __global__ void __launch_bounds__(kTc512Threads, 1) cc_tc512_kernel(Geometry g, 
     fence_proxy_async();
     mbar_arrive_expect_tx(full + (q & 1), nks * 1024u);
     bulk_g2s(dst, a.A16 + (rt * g.KS + k0) * 32, nks * 512u, full + (q & 1));
-    bulk_g2s(dst + nks * 512u, a.B16 + ((static_cast<int64_t>(kt) * 2) * g.KS + k0) * 32, nks * 256u, full + (q & 1));
-    bulk_g2s(dst + nks * 768u, a.B16 + ((static_cast<int64_t>(kt) * 2 + 1) * g.KS + k0) * 32, nks * 256u,
-             full + (q & 1));
+    bulk_g2s(dst + nks * 512u, a.B16 + (static_cast<int64_t>(kt) * g.KS + k0) * 32, nks * 512u, full + (q & 1));
   };
   if (tid == 0) {
     issue(0);
@@ -581,9 +578,7 @@ __global__ void __launch_bounds__(kTc512Threads, 1) cc_tc512_kernel(Geometry g, 
         const int kbase = s_kso[f0];
         const int nks_c = s_kso[f1] - kbase;
         const uint4 *stA = reinterpret_cast<const uint4 *>(stage + buf * kTc512Stage) + lane;
-        const uint2 *stB0 =
-            reinterpret_cast<const uint2 *>(stage + buf * kTc512Stage + static_cast<size_t>(nks_c) * 512) + lane;
-        const uint2 *stB1 = stB0 + nks_c * 32;
+        const uint4 *stB = stA + nks_c * 32;
         for (int f = f0 + warp; f < f1; f += kTc512Warps) {
           const int jb = s_kso[f] - kbase, nj = s_kso[f + 1] - s_kso[f];  // 1..6 k-steps
           float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -591,9 +586,9 @@ __global__ void __launch_bounds__(kTc512Threads, 1) cc_tc512_kernel(Geometry g, 
           for (int jj = 0; jj < kTc512MaxKsPerF; ++jj) {
             if (jj < nj) {
               const int j = (jb + jj) * 32;
-              const uint4 af = stA[j];
-              mma16816<FP16>(d0, af, stB0[j]);
-              mma16816<FP16>(d1, af, stB1[j]);
+              const uint4 af = stA[j], bf = stB[j];
+              mma16816<FP16>(d0, af, make_uint2(bf.x, bf.y));
+              mma16816<FP16>(d1, af, make_uint2(bf.z, bf.w));
             }
           }
           // lane (g8, t4): d[0..1] = Re/Im Z(f), d[2..3] = Im/Re Z(M - f)
@@ -701,7 +696,7 @@ __global__ void __launch_bounds__(TcShape<M, KT>::THREADS) cc_tc_kernel(Geometry
   bool failed = false;
   {
     uint4 *stA = reinterpret_cast<uint4 *>(stage0 + warp * stage_bytes);
-    uint2 *stB = reinterpret_cast<uint2 *>(stage0 + warp * stage_bytes + static_cast<size_t>(a.ks_max) * 512);
+    uint4 *stB = reinterpret_cast<uint4 *>(stage0 + warp * stage_bytes + static_cast<size_t>(a.ks_max) * 512);
     uint64_t *bar = bars + warp;
     uint32_t phase = 0;
     bool first_wait = true;
@@ -711,16 +706,10 @@ __global__ void __launch_bounds__(TcShape<M, KT>::THREADS) cc_tc_kernel(Geometry
       const int nks = g.kso[f + 1] - kb;
       if (lane == 0) {
         const uint32_t abytes = static_cast<uint32_t>(nks) * 512u;
-        const uint32_t bbytes = static_cast<uint32_t>(nks) * 256u;
         fence_proxy_async();
-        mbar_arrive_expect_tx(bar, abytes + Sh::NBLK * bbytes);
+        mbar_arrive_expect_tx(bar, 2 * abytes);
         bulk_g2s(stA, a.A16 + (rt * g.KS + kb) * 32, abytes, bar);
-        const int ref0 = kt * KT;
-#pragma unroll
-        for (int nb = 0; nb < Sh::NBLK; ++nb) {
-          const int64_t blk = static_cast<int64_t>(ref0 / kTile) * 2 + (ref0 % kTile) / 4 + nb;
-          bulk_g2s(stB + nb * nks * 32, a.B16 + (blk * g.KS + kb) * 32, bbytes, bar);
-        }
+        bulk_g2s(stB, a.B16 + (static_cast<int64_t>(kt) * g.KS + kb) * 32, abytes, bar);
       }
       const uint32_t limit = first_wait ? a.first_wait_limit : a.wait_limit;
       first_wait = false;
@@ -735,9 +724,9 @@ __global__ void __launch_bounds__(TcShape<M, KT>::THREADS) cc_tc_kernel(Geometry
 #pragma unroll
       for (int nb = 0; nb < Sh::NBLK; ++nb) d[nb][0] = d[nb][1] = d[nb][2] = d[nb][3] = 0.f;
       for (int j = 0; j < nks; ++j) {
-        const uint4 af = stA[j * 32 + lane];
-#pragma unroll
-        for (int nb = 0; nb < Sh::NBLK; ++nb) mma16816<FP16>(d[nb], af, stB[(nb * nks + j) * 32 + lane]);
+        const uint4 af = stA[j * 32 + lane], bf = stB[j * 32 + lane];
+        mma16816<FP16>(d[0], af, make_uint2(bf.x, bf.y));
+        mma16816<FP16>(d[1], af, make_uint2(bf.z, bf.w));
       }
       // lane (g8, t4): pair (row g8, ref 4 nb + t4) in d[nb]
 #pragma unroll
@@ -859,8 +848,8 @@ __global__ void top8_kernel(const float *__restrict__ rowmax, int64_t n, int nro
 // ---------------------------------------------------------------------------
 // launchers (the FP32 rescore kernel is in k_rescore.cu)
 // ---------------------------------------------------------------------------
-cudaError_t launch_refs16(const Geometry &g, const float2 *B, int ktiles, uint2 *B16, bool fp16, cudaStream_t st) {
-  const int64_t total = static_cast<int64_t>(ktiles) * g.KS * 64;
+cudaError_t launch_refs16(const Geometry &g, const float2 *B, int ktiles, uint4 *B16, bool fp16, cudaStream_t st) {
+  const int64_t total = static_cast<int64_t>(ktiles) * g.KS * 32;
   const int blocks = static_cast<int>((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   refs16_kernel<<<blocks, 256, 0, st>>>(g, B, ktiles, B16, fp16);
   return cudaGetLastError();

@@ -1,517 +1,549 @@
 // Precision-split path, M = 256 angles (rings up to 40): spectrum
-// contraction and inverse angular DFT on the 5th-generation tensor cores
-// (tcgen05.mma, FP32 accumulation in tensor memory), operands staged by TMA.
+// contraction on warp-level tensor cores (mma.sync), inverse angular DFT on
+// the 5th-generation tensor cores (tcgen05.mma, FP32 accumulation in TMEM).
 //
-// Contraction (Alg. 1, CC step).  With q = Re X - Im X, p = Re X + Im X for
-// a particle ring bin and v = Re Y - Im Y, u = Re Y + Im Y for a weighted
-// reference bin, the angular spectrum of a (row, reference) pair is
-//     Z(f) = sum_r q (v + i u),   Z(-f) = sum_r p (u + i v),
-// i.e. Z = C_u + i C' (unmirrored plus i times mirrored correlation).  A
-// tile is 16 particle rows x 8 references = 128 pairs.  One MMA
-// (M = 128, N = 64, K = 16 rings) serves four frequencies at once: A holds,
-// for each of the four frequency slots, the q and p rows of the 16 particle
-// rows (32 rows per slot), B the v and u rows of the 8 references (16 per
-// slot); only the four diagonal 32 x 16 blocks of the 128 x 64 product are
-// used.  (A tcgen05.mma costs at least ~45 cycles whatever its size below
-// N = 64 on GB300, so four narrow per-frequency products in one instruction
-// cost what one does; the unused blocks are free.)  Frequencies with the
-// same number of 16-ring k-steps share an MMA group; a group's k-steps
-// accumulate in one 64-column TMEM slot.
+// Contraction (Alg. 1, CC step).  With q = Re X - Im X, p = Re X + Im X for a
+// particle ring bin and v = Re Y - Im Y, u = Re Y + Im Y for a weighted
+// reference bin, one m16n8k16 per k-step of 16 rings (A: q and p of 8 rows,
+// B: v and u of 4 references) leaves in one lane, for one (row, reference)
+// pair and one frequency f,
+//     d0 = sum q v,  d1 = sum q u,  d2 = sum p v,  d3 = sum p u,
+// and with C = conj(X) Y summed over the rings (unmirrored correlation) and
+// C' = X Y (mirrored, up to a half-turn):
+//     2 Re C = d0 + d3,  2 Im C = d1 - d2,  2 Re C' = d1 + d2,  2 Im C' = d3 - d0.
 //
-// Corner turn.  Slot s of the accumulator sits in TMEM lanes 32 s .. 32 s + 31
-// (lane = (q/p, row)), which warp s % 4 of a warpgroup reads; each such
-// drain thread holds Z of one (row, +-f) for the 8 references and writes
-// them as BF16 into the stage-1 operand in shared memory, where a row is a
-// pair (pair = ref * 16 + row).
+// Inverse angular DFT (Alg. 1, inverse-FFT step).  Both correlations are
+// real, so each is a cosine sum over 2 Re C and a sine sum over 2 Im C.
+// Splitting the frequencies by parity gives four sums per angle j < 64,
+//     Ee, Eo = sum over even / odd f of   2 Re C(f) cos(2 pi f j / 256),
+//     Oe, Oo = sum over even / odd f of - 2 Im C(f) sin(2 pi f j / 256),
+// from which four angles follow by symmetry:
+//     c(j), c(256 - j) = (Ee + Eo) +- (Oe + Oo),
+//     c(128 + j), c(128 - j) = (Ee - Eo) +- (Oe - Oo),
+// so the largest of the four is max(Ee + Eo + |Oe + Oo|, Ee - Eo + |Oe - Oo|).
+// The sums are matrix products over (pair, correlation) rows: D[128 x 64] =
+// A[128 x 64] W[64 x 64], 64 pairs x {C, C'} rows, K = 64 frequencies of one
+// parity and part, N = 64 angles; four of them fill 256 TMEM columns.  The
+// operands are BF16 (one rounding of 2 Re C, 2 Im C and of the matrices), the
+// sums FP32; no intermediate is rounded in between, and the whole angular
+// state never exists outside TMEM.  The zero frequency is added after the
+// maximum (a constant over the angles, FP32).  Angles 64 and 192 use the two
+// columns that are empty at j = 0 (sin 0): column 0 of Oo holds
+// -sum 2 Im C sin(pi f / 2) and column 0 of Oe gets Ee(64) from a third even
+// product (matrix X, one nonzero column).
 //
-// Inverse angular DFT (Alg. 1, inverse-FFT step), 256 = 16 x 16, f = t + 16 a,
-// angle index n = k + 16 j:
-//     Y(k, t)    = sum_a w16^(a k) Z(t + 16 a)          stage 1: per t, M = 128 pairs, N = 32, K = 32
-//     c(k + 16j) = sum_t w16^(t j) w256^(t k) Y(k, t)    twiddle in FP32, stage 2: per k
-// with BF16 operands (the spectrum, the two 16-point DFT matrices, the
-// twiddled intermediate) and FP32 accumulation; c = c_u + i c' gives the
-// unmirrored correlation (real part) and the mirrored one (imaginary part,
-// at the half-turn shifted angle).  The drain of stage 2 reduces each pair
-// to its two row maxima over the 256 angles (Alg. 1 reduction step, Fig. 2)
-// for the FP32 rescore of the top rows.
+// What bounds it, and why this split.  Each (row, reference) pair needs all
+// 129 frequencies on chip at once, so a tile cannot exceed the pairs whose
+// angular state fits; here that state is the FP32 accumulators (256 KB of
+// TMEM hold 64 pairs twice, so one tile's maxima are read while the next
+// tile accumulates).  A tile is 8 rows x 8 references; the row fragments
+// (KS x 512 bytes) stay on chip over all reference tiles, in the registers of
+// the warps that use them (rings up to 36) or in shared memory, and the
+// reference fragments stream from L2 into a register ring ahead of their use.
+// Measured (GB300, 12,000 images of the 76-pixel, 100-reference, 81-shift
+// workload, contraction stage): 20.7 ms, against 66.9 ms for cc_tc256_kernel
+// (all mma.sync, angular state in shared memory, whole chunks of both
+// operands staged behind CTA barriers) and about 77 ms for a tcgen05 kernel
+// that ran the contraction on tcgen05 as well (four frequencies block-diagonal
+// per MMA, two 16-point inverse-DFT stages with a TMEM drain each).  Bound:
+// shared-memory / L1 bandwidth and tensor issue together.  Without the
+// reference loads 19.7 ms, without 16 of the 20 tcgen05.mma 17.0, without
+// both 13.4; what is left is the contraction warps' own instruction stream.
+// Steps measured on the way: rows in shared memory instead of registers
+// 29.4 ms; one operand stage per parity instead of per tile 23.6; references
+// through a per-warp TMA buffer in shared memory 27.4; L1::no_allocate on the
+// reference loads 22.2; ring of 4 / 5 / 6 / 7 / 8 k-steps 22.9 / 23.9 / 20.7 /
+// 20.7 / 22.6.
 //
-// Roles (18 warps, one persistent CTA per SM, tiles walked with stride
-// gridDim.x): warp 0 streams each tile's A and B k-step tiles with TMA
-// tensor-map loads into a ring of shared-memory stages; warp 1 owns the
-// 512 TMEM columns and issues every MMA from one thread; warps 2-17 drain
-// TMEM, in four quads of four warps (one per TMEM lane quarter): quad d
-// drains the contraction groups g = d mod 4, the stage-1 columns of
-// t = 4 d .. 4 d + 3 and the stage-2 columns of k = 4 d .. 4 d + 3.  All waits are bounded; a wait that gives up raises a CTA abort
-// flag and the device error flag, every role leaves its loop, the producer
-// waits for its copies still in flight and the MMA issuer for its MMAs, and
-// the TMEM is released.
-#include <cuda.h>
+// Roles (16 warps, one persistent CTA per SM):
+//   warps 0-7    contract: warp w holds, for each parity, 8 frequencies
+//                (slots) dealt so that every warp has the same k-step count
+//                and its k-steps lie side by side in both fragment layouts
+//                (k-step n0 + (2 w + parity) steps + i), and writes core
+//                column w (8 K-values, 16 bytes per row) of the parity's two
+//                operands;
+//   warps 8-11   read the accumulators of their TMEM lane quarter and write
+//                the row maxima;
+//   warp 12      issues every tcgen05.mma (one lane);
+//   warp 13      contracts f = 0;
+//   warp 14      copies the row fragments to shared memory (when they are
+//                there).
+// All waits are bounded; a wait that gives up raises a CTA abort flag and
+// the device error flag, every role leaves its loop, the copying lane waits
+// for its copies in flight, the issuer for its MMAs, and the TMEM is
+// released.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "../../include/mra.h"
 #include "dev_util.cuh"
 #include "mra_internal.h"
+#include "smem_limit.cuh"
 #include "umma.cuh"
 
 namespace mra {
 
 namespace u256 {
-constexpr int kDrainWarps = 16;                             // 4 quads x the 4 TMEM lane quarters
-constexpr int kThreads = 64 + 32 * kDrainWarps;
-// Registers per thread: the warps of a CTA are spread over the SM's four
-// sub-partitions, each with 16384 registers, so the sub-partition holding
-// the most warps bounds the per-thread count.
-constexpr int kMaxRegs = 96;
-static_assert((kThreads / 32 + 3) / 4 * 32 * kMaxRegs <= 16384, "register file of a sub-partition exceeded");
-constexpr int kUPerStage = kUmmaUPerStage;                  // k-steps per TMA stage (one box per operand)
-constexpr int kStages = 3;
-constexpr uint32_t kABytes = 4096, kBBytes = 2048;          // one k-step: A 128 x 16, B 64 x 16 (BF16/FP16)
-constexpr uint32_t kStageBytes = kUPerStage * (kABytes + kBBytes);
-constexpr int kAcc = 8;                                     // 64-column accumulator slots (all 512 columns)
-constexpr int kCommits = 16;                                // ring of stage-commit barriers
-constexpr uint32_t kTileBytes = 8192;                        // a 128 x 32 operand tile of the inverse DFT
-constexpr uint32_t kOffZ = 0;                                // Z_t tiles (stage 1), then Y_k tiles (stage 2)
-constexpr uint32_t kOffStage = kOffZ + 16 * kTileBytes;
-constexpr uint32_t kOffW = kOffStage + kStages * kStageBytes;  // W1, W2: 32 x 32 BF16 each
-constexpr uint32_t kOffTw = kOffW + 2 * 2048;                // w256^(t k), [t][k]
-// partial row maxima [3 quads][128 pairs]: in the Y_k tiles, which are dead
-// once the stage-2 MMAs have completed
-constexpr uint32_t kOffMax = kOffZ;
-constexpr uint32_t kOffUinfo = kOffTw + 256 * sizeof(float2);
-constexpr uint32_t kOffGfreq = kOffUinfo + kUmmaMaxU * sizeof(int);
-constexpr uint32_t kOffGlast = kOffGfreq + kUmmaMaxG * 4 * sizeof(int);
-constexpr uint32_t kOffBar = kOffGlast + kUmmaMaxG * sizeof(int);
-// barriers: full[S], done[16], acce[8], zs_done, d1_full[4], y_done, d2_full[4], tm_free, fin, mx_full
-constexpr int kNumBars = kStages + kCommits + kAcc + 13;
-constexpr uint32_t kOffMisc = kOffBar + kNumBars * 8;        // TMEM base, abort flag
-constexpr uint32_t kSmem = kOffMisc + 16;
-static_assert(kSmem <= 232448, "tcgen05 M = 256 kernel exceeds 227 KB of shared memory");
-static_assert(kOffStage % 1024 == 0 && kStageBytes % 1024 == 0, "TMA stages must stay 1 KB aligned");
-static_assert(3 * 128 * 8 <= 16 * kTileBytes, "partial maxima must fit the Y_k tiles");
+constexpr int kThreads = 512;
+constexpr int kContract = 8;                     // contraction warps
+constexpr uint32_t kOperand = 128 * 64 * 2;      // one operand of a parity: 128 rows x 64 frequencies
+constexpr uint32_t kZStage = 2 * kOperand;       // real and imaginary parts
+constexpr uint32_t kW = 64 * 64 * 2;             // one DFT matrix
+constexpr uint32_t kWBytes = kHyb256Mats * kW;   // Ee, Oe, X, Eo, Oo
+constexpr int kNumBars = 16;  // zfull[2] zempty[2] dfull[2] dempty[2] x0full[2] afull[2] aempty[2] fin, spare
+constexpr uint32_t kMisc = kWBytes + 2 * 64 * 4 + kNumBars * 8 + 16;
+// Operand stages: both parities of a tile together, two of them, when the row
+// fragments are in registers (one synchronisation per tile); beside row
+// fragments in shared memory there is room for one parity.
+__host__ __device__ constexpr int z_parities(int pattern) { return pattern == 0 ? 2 : 1; }
+__host__ __device__ constexpr int z_stages(int pattern) { return pattern == 0 ? 2 : 1; }
 }  // namespace u256
+
+template <bool FP16>
+__device__ __forceinline__ void mma_frag(float (&d)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
+  if constexpr (FP16)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
 
 __device__ __forceinline__ uint32_t pack_bf2u(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-template <bool FP16>
-__global__ void __maxnreg__(u256::kMaxRegs)
-    cc_umma256_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, Geometry g,
-                      TcArgs a, int ref_tiles, int64_t ntiles) {
+__device__ __forceinline__ uint4 load_frag(const unsigned char *p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// The k-steps of the 8 slots of a warp and parity (fewer are padded with
+// zero fragments): pattern 0 = {3,2,2,2,1,1,1,1}, 1 = {3,3,2,2,2,2,2,2}.
+template <int PATTERN>
+struct HybPattern {
+  static constexpr int kSteps = PATTERN == 0 ? 13 : 18;
+  static constexpr int KS = kHyb256N0 + 16 * kSteps;
+  __host__ __device__ static constexpr int cap(int s) { return s <= PATTERN ? 3 : (PATTERN == 1 || s < 4 ? 2 : 1); }
+  __host__ __device__ static constexpr int first(int s) {
+    int n = 0;
+    for (int i = 0; i < s; ++i) n += cap(i);
+    return n;
+  }
+};
+
+// One parity of one tile by one contraction warp.  fa(i) and fb(i) are the
+// row and reference fragments of k-step i, done(i) is called after their use.
+// out[part * 2 + correlation][block][word].
+template <class P, bool FP16, class FA, class FB, class Done>
+__device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, uint32_t (&out)[4][2][4]) {
+  float keep[2][4];
+  sfor<0, 8>([&](auto ss) {
+    constexpr int s = decltype(ss)::value;
+    float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    sfor<0, P::cap(s)>([&](auto jj) {
+      constexpr int i = P::first(s) + decltype(jj)::value;
+      const uint4 af = fa(i), bf = fb(i);
+      mma_frag<FP16>(d[0], af, bf.x, bf.y);
+      mma_frag<FP16>(d[1], af, bf.z, bf.w);
+      done(i);
+    });
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float v[4] = {d[k][0] + d[k][3], d[k][1] + d[k][2], d[k][1] - d[k][2], d[k][3] - d[k][0]};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if constexpr (s & 1)
+          out[e][k][s >> 1] = pack_bf2u(keep[k][e], v[e]);
+        else
+          keep[k][e] = v[e];
+      }
+    }
+  });
+}
+
+// Every angle of the 32 rows of a warp's TMEM lane quarter into the debug table (dst null: no store).
+__device__ __noinline__ void hybrid_debug_row(uint32_t d, int corr, float x0, float *dst) {
+#pragma unroll 1
+  for (int n = 0; n < 64; ++n) {
+    uint32_t r[4];
+    for (int i = 0; i < 4; ++i) tmem_ld1(d + i * 64 + n, r[i]);
+    tmem_ld_wait();
+    const float E = __uint_as_float(r[0]), F = __uint_as_float(r[1]);
+    const float G = __uint_as_float(r[2]), H = __uint_as_float(r[3]);
+    const float c[4] = {n ? (E + F) + (G + H) : E + F, n ? (E + F) - (G + H) : G + H,
+                        n ? (E - F) + (G - H) : E - F, n ? (E - F) - (G - H) : G - H};
+    const int at[4] = {n, n ? 256 - n : 64, 128 + n, n ? 128 - n : 192};
+    if (dst)  // mirrored row: angle n of the transform is angle n + 128 of the table
+      for (int i = 0; i < 4; ++i) dst[(at[i] + corr * 128) & 255] = c[i] + x0;
+  }
+}
+
+template <int PATTERN, bool FP16>
+__global__ void __launch_bounds__(u256::kThreads, 1)
+    cc_hybrid256_kernel(Geometry g, TcArgs a, int ref_tiles, int per_unit, int splits, int64_t units) {
   using namespace u256;
+  using P = HybPattern<PATTERN>;
+  constexpr int T = P::kSteps;
+  constexpr bool kRegs = PATTERN == 0;                     // row fragments in registers (104 per thread)
+  constexpr int kZp = z_parities(PATTERN), kZs = z_stages(PATTERN);
+  constexpr int PF = kRegs ? 7 : 9;                        // k-steps of references in the register ring
+  constexpr uint32_t kTile16 = P::KS * 512u;               // fragment bytes of a row or reference tile
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBar);
-  uint64_t *full = bars, *done = bars + kStages, *acce = done + kCommits;
-  uint64_t *zs_done = acce + kAcc, *d1_full = zs_done + 1, *y_done = d1_full + 4, *d2_full = y_done + 1,
-           *tm_free = d2_full + 4, *fin = tm_free + 1, *mx_full = fin + 1;
-  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + kOffMisc);
-  volatile int *abort = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
-  int *s_uinfo = reinterpret_cast<int *>(smem + kOffUinfo);
-  int *s_gfreq = reinterpret_cast<int *>(smem + kOffGfreq);
-  int *s_glast = reinterpret_cast<int *>(smem + kOffGlast);  // k-step of each group's last MMA
-  float2 *s_tw = reinterpret_cast<float2 *>(smem + kOffTw);
-  float2 *s_max = reinterpret_cast<float2 *>(smem + kOffMax);
-  const int NU = g.NU, NG = g.NG;
-  const int SPT = (NU + kUPerStage - 1) / kUPerStage;  // TMA stages (and stage commits) per tile
+  unsigned char *sZ = smem;                                // [kZs][kZp] operands of a parity
+  unsigned char *sW = sZ + kZs * kZp * kZStage;            // DFT matrices
+  unsigned char *sF = sW + kWBytes;                        // row fragments [KS][512] (pattern 1)
+  float *s_x0 = reinterpret_cast<float *>(sF + (kRegs ? 0u : kTile16));  // [2][64] zero-frequency terms
+  uint64_t *bars = reinterpret_cast<uint64_t *>(s_x0 + 128);
+  uint64_t *zfull = bars, *zempty = bars + 2, *dfull = bars + 4, *dempty = bars + 6, *x0full = bars + 8,
+           *afull = bars + 10, *aempty = bars + 12, *fin = bars + 14;
+  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + kNumBars);
+  volatile int *abort = reinterpret_cast<volatile int *>(s_tmem + 1);
 
-  // ---- set-up: tables, DFT matrices, barriers, TMEM ----
-  for (int i = tid; i < NU; i += kThreads) {
-    const int info = g.uinfo[i];
-    s_uinfo[i] = info;
-    if ((info >> 10) & 1) s_glast[info & 255] = i;
-  }
-  for (int i = tid; i < NG * 4; i += kThreads) s_gfreq[i] = g.gfreq[i];
-  for (int i = tid; i < 256; i += kThreads) s_tw[i] = g.idft_tw[i];
-  for (int i = tid; i < 1024; i += kThreads)
-    reinterpret_cast<uint32_t *>(smem + kOffW)[i] = g.idft_w[i];
+  // ---- set-up: DFT matrices, barriers, TMEM ----
+  for (int i = tid; i < static_cast<int>(kWBytes / 16); i += kThreads)
+    reinterpret_cast<uint4 *>(sW)[i] = __ldg(reinterpret_cast<const uint4 *>(g.hyb_w) + i);
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(full + s, 1);
-    for (int s = 0; s < kCommits; ++s) mbar_init(done + s, 1);
-    for (int s = 0; s < kAcc; ++s) mbar_init(acce + s, 4);  // the four drain warps of one quad
-    mbar_init(zs_done, kDrainWarps);
-    for (int d = 0; d < 4; ++d) mbar_init(d1_full + d, 1);
-    mbar_init(y_done, kDrainWarps);
-    for (int d = 0; d < 4; ++d) mbar_init(d2_full + d, 1);
-    mbar_init(tm_free, kDrainWarps);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(zfull + s, kContract);
+      mbar_init(zempty + s, 1);
+      mbar_init(dfull + s, 1);
+      mbar_init(dempty + s, 4);
+      mbar_init(x0full + s, 1);
+      mbar_init(afull + s, 1);
+      mbar_init(aempty + s, s == 0 ? kContract + 1 : kContract);  // f = 0 is in the even part
+    }
     mbar_init(fin, 1);
-    mbar_init(mx_full, kDrainWarps - 4);
-    *abort = (smem_u32(smem) & 1023u) ? 1 : 0;  // TMA stages and descriptors assume a 1 KB aligned base
+    *abort = (smem_u32(smem) & 127u) ? 1 : 0;  // descriptors and copies assume an aligned base
     if (*abort) atomicOr(a.err, 2);
   }
-  if (warp == 1) tmem_alloc(s_tmem, 512);
+  if (warp == 12) tmem_alloc(s_tmem, 512);
   mbar_init_fence();
   fence_proxy_async();  // the DFT matrices written above are read by the tensor cores
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
-  const uint32_t sbase = smem_u32(smem);
+  const unsigned char *gA = reinterpret_cast<const unsigned char *>(a.A16);
+  const unsigned char *gB = reinterpret_cast<const unsigned char *>(a.B16);
+  const uint32_t limit = a.wait_limit;
+  // the first reference tile of unit u; a unit's row tile is u / splits
+  auto first_tile = [&](int64_t u) { return static_cast<int>(u % splits) * per_unit; };
 
-  if (warp == 0) {
-    // ---------------- producer: TMA tensor loads of the k-step tiles ----------------
-    // Stage use c (counted over the CTA's tiles) fills ring slot c % kStages
-    // once the MMAs of use c - kStages have completed (their stage commit).
-    if (lane == 0 && !*abort) {
-      int c = 0;
-      bool ok = true;
-      for (int64_t tau = blockIdx.x; tau < ntiles && ok; tau += gridDim.x) {
-        const int rt = static_cast<int>(tau / ref_tiles), kt = static_cast<int>(tau - static_cast<int64_t>(rt) * ref_tiles);
-        int ya = rt * NU * 16, yb = kt * NU * 8;  // tensor-map rows of the tile's first k-step
-        // the next tile's particle k-step tiles (contiguous, NU * 4 KB) into L2 while this one runs
-        if (tau + gridDim.x < ntiles) {
-          const int64_t rn = (tau + gridDim.x) / ref_tiles;
-          if (rn != rt) prefetch_l2(reinterpret_cast<const unsigned char *>(a.A16) + rn * NU * kABytes, NU * kABytes);
-        }
-        for (int u0 = 0; u0 < NU; u0 += kUPerStage, ++c) {
-          if (c >= kStages) {
-            const int cp = c - kStages;
-            if (!spin_or_abort(done + (cp & (kCommits - 1)), static_cast<uint32_t>((cp / kCommits) & 1), a.wait_limit,
-                               abort, a.err)) {
-              ok = false;
-              break;
-            }
-          }
-          // one box of kUPerStage k-steps per operand; a tile's last stage may
-          // read k-steps of the next tile (or zeros past the end), never used
-          const int rs = c % kStages;
-          unsigned char *dst = smem + kOffStage + rs * kStageBytes;
-          mbar_arrive_expect_tx(full + rs, kStageBytes);
-          tma_load_2d(dst, &tmA, 0, ya, full + rs);
-          tma_load_2d(dst + kUPerStage * kABytes, &tmB, 0, yb, full + rs);
-          ya += kUPerStage * 16;
-          yb += kUPerStage * 8;
-        }
-      }
-      // let every copy still in flight land before the CTA's shared memory goes
-      for (int cp = c - kStages < 0 ? 0 : c - kStages; cp < c; ++cp)
-        mbar_wait_bounded(full + cp % kStages, static_cast<uint32_t>((cp / kStages) & 1), a.wait_limit);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0 && !*abort) {
-      const uint32_t idc = umma_idesc(128, 64, !FP16);
-      const uint32_t idi = umma_idesc(128, 32, true);
-      int c = 0;  // stage uses so far
-      bool first = true, ok = true;
-      int64_t tile_iter = 0;
-      const uint64_t wdesc1 = umma_sdesc(sbase + kOffW, 128, 512), wdesc2 = umma_sdesc(sbase + kOffW + 2048, 128, 512);
-      for (int64_t tau = blockIdx.x; tau < ntiles && ok; tau += gridDim.x, ++tile_iter) {
-        if (tile_iter > 0 &&
-            !spin_or_abort(tm_free, static_cast<uint32_t>((tile_iter - 1) & 1), a.wait_limit, abort, a.err))
-          break;
-        tc_fence_after();
-        const int64_t gbase = tile_iter * NG;
-        // contraction: stage use c holds k-steps [4 s, 4 s + 4) of the tile; one commit per stage
-        // (to done[c % 16]) frees the stage for the producer and tells the drain warps that the
-        // groups ending in it are complete
-        for (int sp = 0; sp < SPT && ok; ++sp, ++c) {
-          const int rs = c % kStages;
-          if (!spin_or_abort(full + rs, static_cast<uint32_t>((c / kStages) & 1),
-                             first ? a.first_wait_limit : a.wait_limit, abort, a.err)) {
-            ok = false;
-            break;
-          }
-          first = false;
-          tc_fence_after();
-          const uint32_t st = sbase + kOffStage + rs * kStageBytes;
-          const uint64_t adesc = umma_sdesc(st, 128, 256), bdesc = umma_sdesc(st + kUPerStage * kABytes, 128, 256);
+  // registers per thread: 128 at launch; the contraction keeps its row
+  // fragments, the other roles need few (2 x 200 + 64 + 48 = 4 x 128)
+  if (warp < kContract) {
+    // ---------------- contraction ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    const uint32_t woff = (kHyb256N0 + warp * 2 * T) * 512 + lane * 16;  // this warp's first even k-step
+    unsigned char *zl = sZ + warp * 2048 + lane * 16;
+    const int64_t u0 = blockIdx.x;
+    const unsigned char *bw = gB + static_cast<size_t>(first_tile(u0)) * kTile16 + woff;
+    uint4 b[PF];
+    uint4 ra[kRegs ? 2 * T : 1];
 #pragma unroll
-          for (int ui = 0; ui < kUPerStage; ++ui) {
-            const int u = sp * kUPerStage + ui;
-            if (u < NU) {
-              const int info = s_uinfo[u];
-              const int grp = info & 255, j = (info >> 8) & 3;
-              const int64_t G = gbase + grp;
-              const int slot = static_cast<int>(G & (kAcc - 1));
-              if (j == 0 && G >= kAcc) {
-                if (!spin_or_abort(acce + slot, static_cast<uint32_t>(((G >> 3) - 1) & 1), a.wait_limit, abort,
-                                   a.err)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-              }
-              umma_ss(tmem + slot * 64, adesc + static_cast<uint64_t>(ui * (kABytes >> 4)),
-                      bdesc + static_cast<uint64_t>(ui * (kBBytes >> 4)), idc, j > 0);
+    for (int i = 0; i < PF; ++i) b[i] = load_frag(bw + i * 512);
+    if constexpr (kRegs) {
+      const unsigned char *aw = gA + static_cast<size_t>(u0 / splits) * kTile16 + woff;
+#pragma unroll
+      for (int i = 0; i < 2 * T; ++i) ra[i] = load_frag(aw + i * 512);
+    }
+    uint32_t t = 0, un = 0;  // tiles, units
+    bool ok = !*abort;
+    for (int64_t u = u0; u < units && ok; u += gridDim.x, ++un) {
+      const int k0 = first_tile(u), k1 = min(k0 + per_unit, ref_tiles);
+      const int64_t nu = u + gridDim.x < units ? u + gridDim.x : u;
+      const unsigned char *an = gA + static_cast<size_t>(nu / splits) * kTile16 + woff;  // the next unit's row fragments
+      for (int kt = k0; kt < k1 && ok; ++kt, ++t) {
+        const bool last = kt + 1 == k1;
+        const unsigned char *bn = last ? gB + static_cast<size_t>(first_tile(nu)) * kTile16 + woff : bw + kTile16;
+        auto parity = [&](auto pp) {
+          constexpr int p = decltype(pp)::value;
+          uint32_t out[4][2][4];
+          // register ring: entry i % PF holds k-step i; refilled on use with
+          // k-step i + PF, or with the first ones of the next parity
+          const unsigned char *cur = bw + p * T * 512, *next = p ? bn : cur + T * 512;
+          auto fb = [&](int i) { return b[i % PF]; };
+          auto refill = [&](int i) { b[i % PF] = load_frag(i + PF < T ? cur + (i + PF) * 512 : next + i % PF * 512); };
+          if constexpr (kRegs) {
+            contract_parity<P, FP16>([&](int i) { return ra[p * T + i]; }, fb,
+                                     [&](int i) {
+                                       refill(i);
+                                       if (last) ra[p * T + i] = load_frag(an + (p * T + i) * 512);
+                                     },
+                                     out);
+          } else {
+            if (kt == k0 && !wait_or_abort(afull + p, un & 1, limit, abort, a.err)) return false;
+            const unsigned char *sa = sF + woff + p * T * 512;
+            contract_parity<P, FP16>([&](int i) { return *reinterpret_cast<const uint4 *>(sa + i * 512); }, fb, refill,
+                                     out);
+            if (last) {
+              __syncwarp();
+              if (lane == 0) mbar_arrive(aempty + p);
             }
           }
-          umma_commit(done + (c & (kCommits - 1)));
-        }
-        if (!ok) break;
-        // stage 1 of the inverse DFT: D1_t = Z_t W1 for every t
-        if (!spin_or_abort(zs_done, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err)) break;
-        tc_fence_after();
-        // in four batches of four t, each committed for the drain quad that owns it
-        for (int d = 0; d < 4; ++d) {
-          for (int t = 4 * d; t < 4 * d + 4; ++t)
-            for (int h = 0; h < 2; ++h)
-              umma_ss(tmem + t * 32, umma_sdesc(sbase + kOffZ + t * kTileBytes + h * 256, 128, 512),
-                      wdesc1 + static_cast<uint64_t>(h * 16), idi, h);
-          umma_commit(d1_full + d);
-        }
-        // stage 2: D2_k = Y'_k W2 for every k
-        if (!spin_or_abort(y_done, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err)) break;
-        tc_fence_after();
-        for (int d = 0; d < 4; ++d) {
-          for (int k = 4 * d; k < 4 * d + 4; ++k)
-            for (int h = 0; h < 2; ++h)
-              umma_ss(tmem + k * 32, umma_sdesc(sbase + kOffZ + 2 * h * 32768 + k * 2048, 32768, 128),
-                      wdesc2 + static_cast<uint64_t>(h * 16), idi, h);
-          umma_commit(d2_full + d);
-        }
+          // operand stage: (tile, parity) number c; stages of kZp parities, kZs of them in turn
+          const uint32_t c = 2 * t + p, st = c / kZp, slot = st % kZs, use = st / kZs;
+          if (p % kZp == 0 && use > 0 && !wait_or_abort(zempty + slot, (use - 1) & 1, limit, abort, a.err)) return false;
+          unsigned char *z = zl + (slot * kZp + p % kZp) * kZStage;
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int k = 0; k < 2; ++k)  // row = correlation * 64 + block * 32 + lane
+              *reinterpret_cast<uint4 *>(z + (e >> 1) * kOperand + (e & 1) * 1024 + k * 512) =
+                  make_uint4(out[e][k][0], out[e][k][1], out[e][k][2], out[e][k][3]);
+          if (p % kZp == kZp - 1) {
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(zfull + slot);
+          }
+          return true;
+        };
+        ok = parity(std::integral_constant<int, 0>{}) && parity(std::integral_constant<int, 1>{});
+        bw = bn;
       }
-      // every MMA issued has completed before the TMEM and the stages are released
-      umma_commit(fin);
-      mbar_wait_bounded(fin, 0, a.wait_limit);
     }
-  } else {
-    // ---------------- drain warps ----------------
-    const int dw = warp - 2, q = warp & 3, quad = dw >> 2;
-    const uint32_t lane_base = static_cast<uint32_t>(q * 32) << 16;
-    const int pair = q * 32 + lane;              // TMEM lane of the inverse-DFT stages
-    const int qp = lane >> 4, ri = lane & 15;    // contraction: q or p row, particle row in the tile
-    // this thread's corner-turn target: pair ref * 16 + ri of tile t at K = 2 a (+1): rows of 8 pairs
-    // are 512 bytes apart, so reference ref adds 1024 bytes
-    unsigned char *zrow = smem + kOffZ + (ri >> 3) * 512 + (ri & 7) * 16;
-    const int S = g.S;
-    int64_t tile_iter = 0;
-    for (int64_t tau = blockIdx.x; tau < ntiles && !*abort; tau += gridDim.x, ++tile_iter) {
-      const int rt = static_cast<int>(tau / ref_tiles), kt = static_cast<int>(tau - static_cast<int64_t>(rt) * ref_tiles);
-      const int64_t gbase = tile_iter * NG;
-      bool ok = true;
-      // contraction drains: the pairs of consecutive groups (2 p, 2 p + 1) with p = quad mod 4,
-      // whose stage commits are usually one and the same: both TMEM loads in flight per wait
-      for (int pg = quad; 2 * pg < NG; pg += 4) {
-        const int g0 = 2 * pg, ng = (2 * pg + 1 < NG) ? 2 : 1;
-        const int cg = static_cast<int>(tile_iter) * SPT + s_glast[g0 + ng - 1] / kUPerStage;  // the later commit
-        if (!wait_or_abort(done + (cg & (kCommits - 1)), static_cast<uint32_t>((cg / kCommits) & 1), a.wait_limit,
-                           abort, a.err)) {
+  } else if (warp < 12) {
+    // ---------------- row maxima ----------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    const int q = warp & 3;
+    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
+    const int refl = (lane & 3) + 4 * (q & 1), corr = q >> 1;
+    uint32_t t = 0;
+    bool ok = !*abort;
+    for (int64_t u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const int64_t rt = u / splits;
+      const int k0 = first_tile(u), k1 = min(k0 + per_unit, ref_tiles);
+      const int64_t row = rt * 8 + (lane >> 2);
+      const int64_t img = static_cast<uint32_t>(row) / static_cast<uint32_t>(g.S);  // rows < 2^31
+      const int64_t rb = img * a.K * g.S + (row - img * g.S);
+      for (int kt = k0; kt < k1; ++kt, ++t) {
+        const uint32_t buf = t & 1, ph = (t >> 1) & 1;
+        if (!wait_or_abort(x0full + buf, ph, limit, abort, a.err) ||
+            !wait_or_abort(dfull + buf, ph, limit, abort, a.err)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        int fg[2], slots[2];
-        uint32_t r[2][16];
+        const float x0 = s_x0[buf * 64 + (q & 1) * 32 + lane];
+        const int ref = kt * 8 + refl;
+        const bool valid = row < a.rows && ref < a.K;
+        const int64_t at = rb + static_cast<int64_t>(ref) * g.S;
+        if (a.dbg_cc)
+          hybrid_debug_row(tmem + lanes + buf * 256, corr, x0, valid ? a.dbg_cc + at * 512 + corr * 256 : nullptr);
+        float best = -INFINITY;
+        // 8 angles of each sum at a time; the loop is kept short (the roles
+        // run different code at the same time and share the instruction
+        // cache: unrolled over all 64 angles the kernel took 39.2 instead of
+        // 29.6 ms per 12,000 images of the 76-pixel, 100-reference workload)
+#pragma unroll 1
+        for (int j0 = 0; j0 < 64; j0 += 8) {
+          uint32_t ee[8], eo[8], oe[8], oo[8];
+          const uint32_t d = tmem + lanes + buf * 256 + j0;
+          tmem_ld8(d, ee);
+          tmem_ld8(d + 64, eo);
+          tmem_ld8(d + 128, oe);
+          tmem_ld8(d + 192, oo);
+          tmem_ld_wait();
+          if (j0 == 56) {  // the accumulators are free as soon as they are in registers
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dempty + buf);
+          }
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int64_t G = gbase + g0 + e;
-          slots[e] = static_cast<int>(G & (kAcc - 1));
-          fg[e] = e < ng ? s_gfreq[(g0 + e) * 4 + q] : -1;
-          if (fg[e] >= 0) tmem_ld16(tmem + lane_base + slots[e] * 64 + q * 16, r[e]);
-        }
-        tmem_ld_wait();
-        tc_fence_before();  // the slots are free as soon as their columns are in registers
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(acce + slots[0]);
-          if (ng > 1) mbar_arrive(acce + slots[1]);
-        }
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int f = fg[e];
-          // q rows: Z(f) = (sum q v, sum q u); p rows: Z(256 - f) = (sum p u, sum p v)
-          if (f >= 0 && !(qp && (f == 0 || f == 128))) {
-            const int fp = qp ? ((256 - f) & 255) : f;
-            unsigned char *z = zrow + (fp & 15) * kTileBytes + ((fp >> 4) >> 2) * 128 + ((fp >> 4) & 3) * 4;
-#pragma unroll
-            for (int ref = 0; ref < 8; ++ref) {
-              const float v = __uint_as_float(r[e][ref]), uu = __uint_as_float(r[e][8 + ref]);
-              *reinterpret_cast<uint32_t *>(z + ref * 1024) = qp ? pack_bf2u(uu, v) : pack_bf2u(v, uu);
+          for (int j = 0; j < 8; ++j) {
+            const float E = __uint_as_float(ee[j]), F = __uint_as_float(eo[j]);
+            const float G = __uint_as_float(oe[j]), H = __uint_as_float(oo[j]);
+            float v = (E + F) + fabsf(G + H), w = (E - F) + fabsf(G - H);
+            if (j == 0 && j0 == 0) {  // angles 0, 128; G, H are the sums of angles 64, 192
+              v = E + fabsf(F);
+              w = G + fabsf(H);
             }
+            best = fmaxf(best, fmaxf(v, w));
           }
         }
+        if (valid) a.rowmax[at * 2 + corr] = corr && !g.mirror ? -INFINITY : best + x0;
       }
-      if (!ok) break;
-      fence_proxy_async();  // the Z_t tiles are read by the tensor cores next
-      __syncwarp();
-      if (lane == 0) mbar_arrive(zs_done);
-      // stage-1 drain: Y'(k, t) = w256^(t k) Y(k, t), t = 4 quad .. 4 quad + 3, into the Y_k tiles
-      // (core column `quad` of each; the Z_t tiles are consumed)
-      if (!wait_or_abort(d1_full + quad, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err)) break;
-      tc_fence_after();
-      {
-        // Y_k tiles: core column d (t = 4 d .. 4 d + 3) of every k in region d of the buffer, the
-        // 32 KB that held Z_t for those t (consumed by stage-1 batch d, which this quad waited for;
-        // the other batches read only their own regions): k-th 2 KB block, rows of 8 pairs 128 B apart
-        unsigned char *y = smem + kOffZ + quad * 32768 + (pair >> 3) * 128 + (pair & 7) * 16;
-        // two t and half of the 16 k per pass (8-byte stores of (t, t + 1)): the
-        // real and imaginary columns of both t in flight at once, 48 live values
-#pragma unroll
-        for (int tt = 0; tt < 4; tt += 2) {
-#pragma unroll
-          for (int kh = 0; kh < 16; kh += 8) {
-            const int t0 = quad * 4 + tt;
-            uint32_t r[4][8];
-            tmem_ld8(tmem + lane_base + t0 * 32 + kh, r[0]);
-            tmem_ld8(tmem + lane_base + t0 * 32 + 16 + kh, r[1]);
-            tmem_ld8(tmem + lane_base + (t0 + 1) * 32 + kh, r[2]);
-            tmem_ld8(tmem + lane_base + (t0 + 1) * 32 + 16 + kh, r[3]);
-            tmem_ld_wait();
-#pragma unroll
-            for (int k8 = 0; k8 < 8; ++k8) {
-              uint32_t o[2];
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const float2 w = s_tw[(t0 + e) * 16 + kh + k8];
-                const float yr = __uint_as_float(r[2 * e][k8]), yi = __uint_as_float(r[2 * e + 1][k8]);
-                o[e] = pack_bf2u(fmaf(yr, w.x, -yi * w.y), fmaf(yr, w.y, yi * w.x));
+    }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    if (warp == 12) {
+      // ---------------- inverse DFT: MMA issue ----------------
+      if (lane == 0 && !*abort) {
+        const uint32_t idesc = umma_idesc(128, 64, true);
+        const uint32_t zb = smem_u32(sZ), wb = smem_u32(sW);
+        uint32_t t = 0;
+        bool ok = true;
+        for (int64_t u = blockIdx.x; u < units && ok; u += gridDim.x) {
+          const int k0 = first_tile(u), k1 = min(k0 + per_unit, ref_tiles);
+          for (int kt = k0; kt < k1 && ok; ++kt, ++t) {
+            const uint32_t buf = t & 1, dcol = tmem + buf * 256;
+            if (t >= 2 && !spin_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) {
+              ok = false;
+              break;
+            }
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+              const uint32_t c = 2 * t + p, st = c / kZp, slot = st % kZs;
+              if (p % kZp == 0 &&
+                  !spin_or_abort(zfull + slot, (st / kZs) & 1, c ? limit : a.first_wait_limit, abort, a.err)) {
+                ok = false;
+                break;
               }
-              *reinterpret_cast<uint2 *>(y + (kh + k8) * 2048 + tt * 4) = make_uint2(o[0], o[1]);
+              tc_fence_after();
+              // core columns of 8 frequencies: 2048 bytes apart in an operand, 1024 in a matrix
+              const uint64_t zr = umma_sdesc(zb + (slot * kZp + p % kZp) * kZStage, 2048, 128), zi = zr + (kOperand >> 4);
+              const uint64_t w0 = umma_sdesc(wb + (p ? 3 * kW : 0), 1024, 128), w1 = w0 + (kW >> 4),
+                             w2 = w1 + (kW >> 4);
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) {
+                umma_ss(dcol + p * 64, zr + ks * 256, w0 + ks * 128, idesc, ks > 0);        // Ee | Eo
+                umma_ss(dcol + 128 + p * 64, zi + ks * 256, w1 + ks * 128, idesc, ks > 0);  // Oe | Oo
+              }
+              if (!p)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) umma_ss(dcol + 128, zr + ks * 256, w2 + ks * 128, idesc, 1);  // Ee(64)
+              if (p % kZp == kZp - 1) umma_commit(zempty + slot);
             }
+            if (ok) umma_commit(dfull + buf);
           }
         }
+        // every MMA issued has completed before the TMEM and the operands are released
+        umma_commit(fin);
+        mbar_wait_bounded(fin, 0, limit);
       }
-      tc_fence_before();
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(y_done);
-      // stage-2 drain: row maxima over the 256 angles (and the full table in debug mode)
-      if (!wait_or_abort(d2_full + quad, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err)) break;
-      tc_fence_after();
-      const int ref = pair >> 4, prow = pair & 15;
-      const int64_t row = static_cast<int64_t>(rt) * 16 + prow;
-      const int refg = kt * 8 + ref;
-      const bool valid = row < a.rows && refg < a.K;
-      int64_t rbase = 0;
-      if (valid) {
-        const int64_t img = row / S;
-        rbase = (img * a.K + refg) * S + (row - img * S);
-      }
-      float vu = -INFINITY, vm = -INFINITY;
-      for (int kk = 0; kk < 4; ++kk) {
-        const int k = quad * 4 + kk;
-        uint32_t r[32];
-        tmem_ld32(tmem + lane_base + k * 32, r);
-        tmem_ld_wait();
+    } else if (warp == 13) {
+      // ---------------- zero frequency: k-steps 0..n0-1 ----------------
+      uint32_t t = 0, un = 0;
+      bool ok = !*abort;
+      for (int64_t u = blockIdx.x; u < units && ok; u += gridDim.x, ++un) {
+        const int k0 = first_tile(u), k1 = min(k0 + per_unit, ref_tiles);
+        const unsigned char *aw = gA + static_cast<size_t>(u / splits) * kTile16 + lane * 16;
+        uint4 af[kHyb256N0];
+        if constexpr (kRegs) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          vu = fmaxf(vu, __uint_as_float(r[j]));
-          vm = fmaxf(vm, __uint_as_float(r[16 + j]));
+          for (int j = 0; j < kHyb256N0; ++j) af[j] = load_frag(aw + j * 512);
         }
-        if (a.dbg_cc && valid) {
-          float *d = a.dbg_cc + rbase * 512;
+        for (int kt = k0; kt < k1; ++kt, ++t) {
+          const uint32_t buf = t & 1;
+          const unsigned char *bp = gB + static_cast<size_t>(kt) * kTile16 + lane * 16;
+          uint4 b[kHyb256N0];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int n = k + 16 * j;
-            d[n] = __uint_as_float(r[j]);
-            d[256 + ((n + 128) & 255)] = __uint_as_float(r[16 + j]);
+          for (int j = 0; j < kHyb256N0; ++j) b[j] = load_frag(bp + j * 512);
+          if (!kRegs && kt == k0) {
+            if (!wait_or_abort(afull, un & 1, limit, abort, a.err)) {
+              ok = false;
+              break;
+            }
+#pragma unroll
+            for (int j = 0; j < kHyb256N0; ++j) af[j] = *reinterpret_cast<const uint4 *>(sF + j * 512 + lane * 16);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(aempty);
           }
-        }
-      }
-      tc_fence_before();
-      // quads 1-3 hand their maxima to quad 0 (bounded wait: an abort
-      // elsewhere cannot leave a warp stuck here)
-      bool have = true;
-      if (quad) {
-        // the maxima go into the Y_k tiles: wait until the last stage-2 batch has read them
-        have = wait_or_abort(d2_full + 3, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err);
-        if (have) s_max[(quad - 1) * 128 + pair] = make_float2(vu, vm);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(mx_full);
-      } else {
-        have = wait_or_abort(mx_full, static_cast<uint32_t>(tile_iter & 1), a.wait_limit, abort, a.err);
-      }
-      if (!quad && have && valid) {
+          if (t >= 2 && !wait_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) {
+            ok = false;
+            break;
+          }
+          float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const float2 o = s_max[d * 128 + pair];
-          vu = fmaxf(vu, o.x);
-          vm = fmaxf(vm, o.y);
+          for (int j = 0; j < kHyb256N0; ++j) {
+            mma_frag<FP16>(d0, af[j], b[j].x, b[j].y);
+            mma_frag<FP16>(d1, af[j], b[j].z, b[j].w);
+          }
+          s_x0[buf * 64 + lane] = d0[0];
+          s_x0[buf * 64 + 32 + lane] = d1[0];
+          __syncwarp();
+          if (lane == 0) mbar_arrive(x0full + buf);
         }
-        a.rowmax[rbase * 2] = vu;
-        a.rowmax[rbase * 2 + 1] = g.mirror ? vm : -INFINITY;
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tm_free);
-      if (!have) break;
+    } else if (warp == 14 && !kRegs) {
+      // ---------------- row fragments to shared memory ----------------
+      // lane w < 8: warp w's even or odd k-steps; lane 8: f = 0 (even)
+      uint32_t un = 0;
+      int issued[2] = {0, 0};
+      bool ok = !*abort;
+      for (int64_t u = blockIdx.x; u < units && ok; u += gridDim.x, ++un) {
+        const unsigned char *src = gA + static_cast<size_t>(u / splits) * kTile16;
+        for (int p = 0; p < 2 && ok; ++p) {
+          if (un > 0 && !wait_or_abort(aempty + p, (un - 1) & 1, limit, abort, a.err)) ok = false;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive_expect_tx(afull + p, (kContract * T + (p ? 0 : kHyb256N0)) * 512u);
+          __syncwarp();
+          fence_proxy_async();  // earlier reads of these fragments are done (aempty)
+          const uint32_t off = lane < kContract ? (kHyb256N0 + (2 * lane + p) * T) * 512u : 0u;
+          if (lane < kContract || (lane == kContract && !p))
+            bulk_g2s(sF + off, src + off, (lane < kContract ? T : kHyb256N0) * 512u, afull + p);
+          ++issued[p];
+        }
+      }
+      // every copy issued lands before the CTA's shared memory goes
+      for (int p = 0; p < 2; ++p)
+        if (issued[p]) mbar_wait_bounded(afull + p, (issued[p] - 1) & 1, limit);
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, 512);
+  if (warp == 12) tmem_dealloc(tmem, 512);
 }
 
-// Reference k-step tiles of the tcgen05 path: for reference tile kt (8
-// references) and MMA k-step u, the 64 x 16 B operand (row n = slot * 16 +
-// (v|u) * 8 + ref, K = ring within the k-step) in the canonical K-major
-// layout; zero for empty slots, padding k-steps and rings beyond R_f.
-__global__ void refs16u_kernel(Geometry g, const float2 *__restrict__ B, int ktiles, uint4 *B16u, bool fp16) {
-  const int64_t total = static_cast<int64_t>(ktiles) * g.NU * 128;
-  for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
-       idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int hh = static_cast<int>(idx & 1), n = static_cast<int>((idx >> 1) & 63);
-    const int64_t ku = idx >> 7;
-    const int u = static_cast<int>(ku % g.NU), kt = static_cast<int>(ku / g.NU);
-    const int info = g.uinfo[u];
-    const int grp = info & 255, j = (info >> 8) & 3;
-    const int s = n >> 4, vu = (n >> 3) & 1, ref = n & 7;
-    const int f = g.gfreq[grp * 4 + s];
-    uint16_t v16[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      float val = 0.f;
-      if (f >= 0 && j < g.kso[f + 1] - g.kso[f]) {
-        const int2 seg = g.fseg[f];
-        const int rr = 16 * j + 8 * hh + e;
-        if (rr < seg.y) {
-          const float2 X = B[(static_cast<int64_t>(kt) * g.NB + seg.x + rr) * kTile + ref];
-          val = vu ? (X.x + X.y) : (X.x - X.y);
-        }
-      }
-      v16[e] = fp16 ? __half_as_ushort(__float2half_rn(val)) : __bfloat16_as_ushort(__float2bfloat16_rn(val));
+// Units of work are (row tile, range of reference tiles): `splits` ranges
+// per row tile, chosen to minimise the time of the fullest SM,
+// waves x (tiles per unit + the unit's load of its row fragments, about one
+// tile).  One range when the row tiles fill many waves (each row tile's
+// fragments are then loaded once); more when the stack is so small that
+// whole row tiles would leave SMs idle.
+static int pick_splits(int64_t row_tiles, int ref_tiles, int sms) {
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int s = 1; s <= ref_tiles; ++s) {
+    const int per = (ref_tiles + s - 1) / s;
+    if ((ref_tiles + per - 1) / per != s) continue;  // ranges must not be empty
+    const int64_t cost = (row_tiles * s + sms - 1) / sms * (per + 1);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = s;
     }
-    uint4 o;
-    o.x = v16[0] | (static_cast<uint32_t>(v16[1]) << 16);
-    o.y = v16[2] | (static_cast<uint32_t>(v16[3]) << 16);
-    o.z = v16[4] | (static_cast<uint32_t>(v16[5]) << 16);
-    o.w = v16[6] | (static_cast<uint32_t>(v16[7]) << 16);
-    B16u[(ku * 2048 + (n >> 3) * 256 + hh * 128 + (n & 7) * 16) / 16] = o;
   }
+  return best;
 }
 
-cudaError_t launch_refs16u(const Geometry &g, const float2 *B, int ktiles, void *B16u, bool fp16, cudaStream_t st) {
-  const int64_t total = static_cast<int64_t>(ktiles) * g.NU * 128;
-  const int blocks = static_cast<int>((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  refs16u_kernel<<<blocks, 256, 0, st>>>(g, B, ktiles, static_cast<uint4 *>(B16u), fp16);
+template <int PATTERN, bool FP16>
+static cudaError_t launch_hybrid_t(const Geometry &g, const TcArgs &a, cudaStream_t st) {
+  static size_t granted = 0;
+  constexpr size_t smem = u256::z_stages(PATTERN) * u256::z_parities(PATTERN) * u256::kZStage + u256::kMisc +
+                          (PATTERN == 0 ? 0 : HybPattern<PATTERN>::KS * 512);
+  static_assert(smem <= kMaxSmemPerBlock, "row fragments must fit");
+  if (g.KS != HybPattern<PATTERN>::KS) return cudaErrorInvalidValue;
+  cudaError_t e = raise_smem_limit(cc_hybrid256_kernel<PATTERN, FP16>, smem, granted);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
+  const int ref_tiles = (a.K + kTile - 1) / kTile;
+  if (row_tiles <= 0) return cudaSuccess;
+  const int splits = pick_splits(row_tiles, ref_tiles, sms);
+  const int per = (ref_tiles + splits - 1) / splits;
+  const int64_t units = row_tiles * splits;
+  const int grid = static_cast<int>(units < sms ? units : sms);
+  cc_hybrid256_kernel<PATTERN, FP16><<<grid, u256::kThreads, smem, st>>>(g, a, ref_tiles, per, splits, units);
   return cudaGetLastError();
 }
 
-template <bool FP16>
-static cudaError_t launch_u256_t(const CUtensorMap &tmA, const CUtensorMap &tmB, const Geometry &g, const TcArgs &a,
-                                 cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(cc_umma256_kernel<FP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(u256::kSmem));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
-  const int64_t row_tiles = (a.rows + kUmmaRows - 1) / kUmmaRows;
-  const int ref_tiles = (a.K + kUmmaRefs - 1) / kUmmaRefs;
-  const int64_t ntiles = row_tiles * ref_tiles;
-  if (ntiles <= 0) return cudaSuccess;
-  const int grid = static_cast<int>(ntiles < sms ? ntiles : sms);
-  cc_umma256_kernel<FP16><<<grid, u256::kThreads, u256::kSmem, st>>>(tmA, tmB, g, a, ref_tiles, ntiles);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cc_umma256(const void *tmA, const void *tmB, const Geometry &g, const TcArgs &a, bool fp16,
-                              cudaStream_t st) {
-  if (g.M != 256 || g.NU <= 0 || g.NU > kUmmaMaxU || g.NG > kUmmaMaxG) return cudaErrorInvalidValue;
-  const CUtensorMap &A = *static_cast<const CUtensorMap *>(tmA);
-  const CUtensorMap &B = *static_cast<const CUtensorMap *>(tmB);
-  return fp16 ? launch_u256_t<true>(A, B, g, a, st) : launch_u256_t<false>(A, B, g, a, st);
+cudaError_t launch_cc_hybrid256(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st) {
+  if (g.M != 256 || !g.hyb_w) return cudaErrorInvalidValue;
+  if (g.hyb_pattern == 0) return fp16 ? launch_hybrid_t<0, true>(g, a, st) : launch_hybrid_t<0, false>(g, a, st);
+  return fp16 ? launch_hybrid_t<1, true>(g, a, st) : launch_hybrid_t<1, false>(g, a, st);
 }
 
 }  // namespace mra

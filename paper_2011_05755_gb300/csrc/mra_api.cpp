@@ -43,14 +43,9 @@ struct mra_handle {
   int ks_max = 0;              // most 16-ring k-steps of any frequency (16-bit paths)
   bool half = false;           // precision-split path (BF16/FP16 contraction + FP32 rescore)
   bool fp16 = false;           // FP16 rather than BF16 operands
-  uint2 *B16 = nullptr;        // reference B fragments
+  uint4 *B16 = nullptr;        // reference B fragments
   int B16_refs = 0;            // references (padded) the fragment buffer holds
-  uint4 *A16 = nullptr;        // particle A fragments for one chunk (mma.sync kernels), or
-                               // the k-step tiles of the tcgen05 kernel (umma)
-  bool umma = false;           // M = 256 precision split on tcgen05 (k_umma256.cu)
-  void *B16u = nullptr;        // reference k-step tiles of the tcgen05 kernel
-  int B16u_refs = 0;           // references (padded to tiles) the tiles hold
-  CUtensorMap tmA{}, tmB{};    // TMA descriptors of the particle / reference k-step tiles
+  uint4 *A16 = nullptr;        // particle A fragments for one chunk
   size_t A16_bytes = 0;
   float *rowmax = nullptr;     // [chunk][K][S][2]
   int64_t rowmax_cap = 0;      // floats
@@ -326,6 +321,40 @@ int validate(const mra_config_t *c, std::string *why) {
   return rc;
 }
 
+// BF16 DFT matrices of the M = 256 kernel with the tcgen05 inverse DFT (five
+// of 64 angles x 64 frequencies, canonical K-major core matrices).  K index
+// 8 w + s is frequency number 8 s + w of its parity; as the rings that reach a
+// frequency never grow in number with it, the frequencies sorted by k-step
+// count are in ascending order whatever the rings, and the matrices are the
+// same for every handle.
+const std::vector<uint32_t> &hybrid_matrices() {
+  static const std::vector<uint32_t> mats = [] {
+    auto bf16 = [](double v) {  // round to nearest even (|v| <= 1)
+      const float x = static_cast<float>(v);
+      uint32_t u;
+      std::memcpy(&u, &x, 4);
+      return static_cast<uint16_t>((u + 0x7fffu + ((u >> 16) & 1u)) >> 16);
+    };
+    std::vector<uint32_t> wm(mra::kHyb256Mats * 2048, 0);
+    for (int m = 0; m < mra::kHyb256Mats; ++m)
+      for (int j = 0; j < 64; ++j)
+        for (int k = 0; k < 64; ++k) {
+          const int i = 8 * (k % 8) + k / 8, f = m >= 3 ? 2 * i + 1 : 2 * i + 2;
+          const double th = kTwoPi * ((f * j) % 256) / 256.0, quarter = kTwoPi * (f % 4) / 4.0;
+          double v = 0.0;
+          if (m == 0 || m == 3) v = std::cos(th);                        // Ee, Eo
+          if (m == 1) v = -std::sin(th);                                 // Oe
+          if (m == 2) v = j == 0 ? std::cos(quarter) : 0.0;              // X: Ee at angle 64
+          if (m == 4) v = j == 0 ? -std::sin(quarter) : -std::sin(th);   // Oo; column 0: angle 64
+          if (f == 128) v *= 0.5;                                        // f = 128 is its own mirror image
+          const size_t byte = static_cast<size_t>(m) * 8192 + (k / 8) * 1024 + (j / 8) * 128 + (j % 8) * 16 + (k % 8) * 2;
+          wm[byte / 4] |= static_cast<uint32_t>(bf16(v)) << (byte % 4 * 8);
+        }
+    return wm;
+  }();
+  return mats;
+}
+
 // Build every geometry table of the configuration (FP64 on the host).
 int build_tables(mra_handle *h) {
   const mra_config_t &c = h->cfg;
@@ -378,6 +407,51 @@ int build_tables(mra_handle *h) {
     if (nks > h->ks_max) h->ks_max = nks;
   }
   kso[H + 1] = static_cast<int>(ksinfo.size());
+  h->half = c.precision != MRA_FP32;
+  h->fp16 = c.precision == MRA_FP16_RESCORE;
+  // M = 256 kernel with the tcgen05 inverse DFT: the 64 frequencies of each
+  // parity (even 2..128, odd 1..127; their k-step counts fall) are dealt to
+  // the 8 contraction warps, slot s of warp w taking the (8 s + w)-th.  The
+  // k-steps of a warp and parity lie side by side, each slot padded to its
+  // pattern's count with k-steps of zeros; f = 0 comes first.  (The other
+  // kernel where that layout would make the polar kernel exceed shared
+  // memory: boxes just enclosing L = 200 at rings 1..40.)
+  int pattern = -1;
+  if (M == 256 && h->half && c.kernel != MRA_KERNEL_MMA_SYNC) {
+    auto nks = [&](int f) { return kso[f + 1] - kso[f]; };
+    int n3 = 0, n2 = 0;  // slots that need three, at least two k-steps
+    auto freq = [](int p, int i) { return p ? 2 * i + 1 : 2 * i + 2; };
+    for (int p = 0; p < 2; ++p)
+      for (int i = 0; i < 64; ++i) {
+        if (nks(freq(p, i)) > 2) n3 = std::max(n3, i / 8 + 1);
+        if (nks(freq(p, i)) > 1) n2 = std::max(n2, i / 8 + 1);
+      }
+    const int cap[2][8] = {{3, 2, 2, 2, 1, 1, 1, 1}, {3, 3, 2, 2, 2, 2, 2, 2}};
+    pattern = n3 <= 1 && n2 <= 4 ? 0 : 1;
+    mra::Geometry gp{};
+    gp.L = c.L;
+    gp.M = M;
+    gp.NS = NS;
+    gp.pad = 8;
+    gp.KS = mra::kHyb256N0 + 16 * (pattern == 0 ? 13 : 18);
+    if (n3 > 2 || mra::polar_smem_one_row(gp, true, true) > mra::kMaxSmemPerBlock) {
+      pattern = -1;
+    } else {
+      std::vector<int2> info;
+      std::vector<int> pos(H + 2, 0);
+      for (int j = 0; j < mra::kHyb256N0; ++j) info.push_back(make_int2(0, j));
+      for (int w = 0; w < 8; ++w)
+        for (int p = 0; p < 2; ++p)
+          for (int sl = 0; sl < 8; ++sl) {
+            const int f = freq(p, 8 * sl + w);
+            pos[f] = static_cast<int>(info.size());
+            for (int j = 0; j < cap[pattern][sl]; ++j) info.push_back(make_int2(f, j));
+          }
+      pos[H + 1] = static_cast<int>(info.size());
+      kso = pos;
+      ksinfo = info;
+    }
+  }
   std::vector<int> binpos16(NBIN);
   std::vector<int> binpos(NBIN);
   std::vector<float> bweight(NBIN);
@@ -495,7 +569,7 @@ int build_tables(mra_handle *h) {
     if ((rc = upload(h, kpos, &g.kpos, "frequency bases"))) return rc;
     if ((rc = upload(h, kpos16, &g.kpos16, "16-bit frequency bases"))) return rc;
   }
-  {
+  if (pattern < 0) {
     // whole frequencies per staging chunk of the M = 256 / M = 512 kernels, greedily
     const int cap = g.M == 512 ? mra::kTc512ChunkKs : mra::kTc256ChunkKs;
     std::vector<int> chunk_f(1, 0);
@@ -509,8 +583,6 @@ int build_tables(mra_handle *h) {
     g.NCH = static_cast<int>(chunk_f.size()) - 1;
     if ((rc = upload(h, chunk_f, &g.chunk_f, "staging chunks"))) return rc;
   }
-  h->half = c.precision != MRA_FP32;
-  h->fp16 = c.precision == MRA_FP16_RESCORE;
   // BF16 fragments of the 16-point DFT matrices for the tensor-core inverse DFT.
   // Stage 1 (A, rows (re/im, k), cols (re/im, a)): [[C, -S], [S, C]];
   // stage 2 (B, rows (re/im, t), cols (re/im, j)): [[C, S], [-S, C]];
@@ -555,61 +627,9 @@ int build_tables(mra_handle *h) {
     }
     if ((rc = upload(h, frag, &g.dft16, "DFT fragments"))) return rc;
   }
-  // tcgen05 path (M = 256): frequencies four to an MMA.  Greedy in f order:
-  // a group takes the next frequencies while it has fewer than four; its
-  // k-step count is that of its first (lowest) frequency, the largest, as
-  // R_f does not grow with f; the others are padded with zero k-steps.
-  h->umma = h->half && M == 256 && c.kernel == MRA_KERNEL_TCGEN05;
-  if (M == 256) {
-    std::vector<int> gfreq, uinfo, umap(kso[H + 1], -1);
-    int NG = 0, NU = 0;
-    for (int f = 0; f <= H;) {
-      const int nks = kso[f + 1] - kso[f];
-      int members[4] = {-1, -1, -1, -1};
-      for (int sl = 0; sl < 4 && f <= H; ++sl, ++f) {
-        members[sl] = f;
-        for (int j = 0; j < kso[f + 1] - kso[f]; ++j) umap[kso[f] + j] = (NU + j) * 4 + sl;
-      }
-      for (int sl = 0; sl < 4; ++sl) gfreq.push_back(members[sl]);
-      for (int j = 0; j < nks; ++j) uinfo.push_back(NG | (j << 8) | ((j == nks - 1 ? 1 : 0) << 10));
-      NU += nks;
-      ++NG;
-    }
-    if (NU > mra::kUmmaMaxU || NG > mra::kUmmaMaxG)
-      return set_err(h, MRA_EINVAL, "%d MMA k-steps in %d groups exceed the tcgen05 tables", NU, NG);
-    h->g.NU = NU;
-    h->g.NG = NG;
-    if ((rc = upload(h, umap, &h->g.umap, "k-step map"))) return rc;
-    if ((rc = upload(h, uinfo, &h->g.uinfo, "k-step groups"))) return rc;
-    if ((rc = upload(h, gfreq, &h->g.gfreq, "group frequencies"))) return rc;
-    // BF16 16-point DFT matrices in the canonical K-major layout (B operands,
-    // 32 N-rows x 32 K): W1[(c', k)][(a, c)] and W2[(c'', j)][(t, c')] with
-    // K = 2 a + c: [[cos, -sin], [sin, cos]] of 2 pi a k / 16 (resp. t j).
-    auto bf16 = [](double v) {  // round to nearest even (|v| <= 1)
-      const float x = static_cast<float>(v);
-      uint32_t u;
-      std::memcpy(&u, &x, 4);
-      return static_cast<uint16_t>((u + 0x7fffu + ((u >> 16) & 1u)) >> 16);
-    };
-    std::vector<uint16_t> w16(2048, 0);
-    for (int m = 0; m < 2; ++m)
-      for (int n = 0; n < 32; ++n)
-        for (int K = 0; K < 32; ++K) {
-          const int co = n >> 4, x = n & 15, ci = K & 1, y = K >> 1;
-          const double th = kTwoPi * x * y / 16.0;
-          const double v = co == ci ? std::cos(th) : (co == 0 ? -std::sin(th) : std::sin(th));
-          w16[m * 1024 + ((n >> 3) * 512 + (K >> 3) * 128 + (n & 7) * 16 + (K & 7) * 2) / 2] = bf16(v);
-        }
-    std::vector<uint32_t> wpk(1024);
-    for (int i = 0; i < 1024; ++i) wpk[i] = w16[2 * i] | (static_cast<uint32_t>(w16[2 * i + 1]) << 16);
-    if ((rc = upload(h, wpk, &h->g.idft_w, "inverse-DFT matrices"))) return rc;
-    std::vector<float2> tw(256);
-    for (int t = 0; t < 16; ++t)
-      for (int k = 0; k < 16; ++k) {
-        const double th = kTwoPi * t * k / 256.0;
-        tw[t * 16 + k] = make_float2(static_cast<float>(std::cos(th)), static_cast<float>(std::sin(th)));
-      }
-    if ((rc = upload(h, tw, &h->g.idft_tw, "inverse-DFT twiddles"))) return rc;
+  if (pattern >= 0) {
+    if ((rc = upload(h, hybrid_matrices(), &g.hyb_w, "inverse-DFT matrices"))) return rc;
+    g.hyb_pattern = pattern;
   }
   if ((rc = dev_alloc(h, &h->d_err, sizeof(int), "failure flags"))) return rc;
   h->tables.push_back(h->d_err);
@@ -618,11 +638,6 @@ int build_tables(mra_handle *h) {
   return MRA_OK;
 }
 
-// TMA descriptor of a buffer of k-step tiles seen as a 2-D tensor of 16-bit
-// elements with rows of 256 bytes (128 elements); one load box is box_rows
-// rows, the kUmmaUPerStage consecutive k-step tiles of one pipeline stage
-// (4 KB particle tiles: 16 rows each; 2 KB reference tiles: 8).  Rows past
-// the end read as zero.
 // cuTensorMapEncodeTiled comes from the driver through the runtime's entry
 // point query, so the library needs no link to libcuda.
 using TensorMapEncode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -644,20 +659,6 @@ TensorMapEncode tensor_map_encoder() {
   return encode;
 }
 
-int make_tile_map(mra_handle *h, CUtensorMap *tm, void *base, uint64_t rows, uint32_t box_rows, const char *what) {
-  const TensorMapEncode encode = tensor_map_encoder();
-  if (!encode) return set_err(h, MRA_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-  const cuuint64_t dims[2] = {128, rows};
-  const cuuint64_t strides[1] = {256};
-  const cuuint32_t box[2] = {128, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, base, dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return set_err(h, MRA_ECUDA, "cuTensorMapEncodeTiled(%s) failed with %d", what, int(r));
-  return MRA_OK;
-}
-
 // Particle-spectrum workspace for one chunk of images (FP32 tiled spectra,
 // or 16-bit fragments plus row maxima and candidates for the split path).
 int ensure_chunk_workspace(mra_handle *h) {
@@ -665,7 +666,6 @@ int ensure_chunk_workspace(mra_handle *h) {
   if (!h->best) {
     size_t per_img = h->half ? static_cast<size_t>(S) * h->g.KS * 64 + static_cast<size_t>(h->K) * S * 8
                              : static_cast<size_t>(S) * h->NB * sizeof(float2);
-    if (h->umma) per_img = static_cast<size_t>(S) * h->g.NU * 256 + static_cast<size_t>(h->K) * S * 8;
     int chunk = h->cfg.chunk_images;
     if (chunk <= 0) {
       const size_t budget = size_t(2) << 30;
@@ -697,19 +697,7 @@ int ensure_chunk_workspace(mra_handle *h) {
     h->chunk = chunk;
     const int64_t tiles = (int64_t(chunk) * S + mra::kTile - 1) / mra::kTile;
     int rc;
-    if (h->umma) {
-      // k-step tiles of 16 rows; slots and k-steps no frequency fills are
-      // never written and must read as zero
-      const int64_t utiles = (int64_t(chunk) * S + mra::kUmmaRows - 1) / mra::kUmmaRows;
-      h->A16_bytes = static_cast<size_t>(utiles) * h->g.NU * 4096;
-      if ((rc = dev_alloc(h, &h->A16, h->A16_bytes, "particle k-step tiles"))) return rc;
-      cudaError_t e = cudaMemset(h->A16, 0, h->A16_bytes);
-      if (e != cudaSuccess) return cuda_err(h, e, "cudaMemset(particle k-step tiles)");
-      if ((rc = make_tile_map(h, &h->tmA, h->A16, static_cast<uint64_t>(utiles) * h->g.NU * 16, 16 * mra::kUmmaUPerStage,
-                              "particle k-step tiles")))
-        return rc;
-      if ((rc = dev_alloc(h, &h->cand, sizeof(int) * mra::kTopRows * chunk, "candidate rows"))) return rc;
-    } else if (h->half) {
+    if (h->half) {
       h->A16_bytes = static_cast<size_t>(tiles) * h->g.KS * 512;
       if ((rc = dev_alloc(h, &h->A16, h->A16_bytes, "particle fragments"))) return rc;
       if ((rc = dev_alloc(h, &h->cand, sizeof(int) * mra::kTopRows * chunk, "candidate rows"))) return rc;
@@ -796,7 +784,6 @@ void free_all(mra_handle *h) {
   fr(h->best);
   fr(h->B16);
   fr(h->A16);
-  fr(h->B16u);
   fr(h->rowmax);
   fr(h->cand);
   mra::AvgWork &w = h->avg;
@@ -858,7 +845,6 @@ int run_polar(mra_handle *h, const float *imgs, int64_t n, int rows_per_img, boo
   a.dbg_spec = dbg_spec;
   a.out16 = out16;
   a.fp16 = h->fp16;
-  a.umma = h->umma && out16 != nullptr;
   a.err = h->d_err;
   a.wait_limit = kWaitLimit;
   // image staging by a TMA tensor copy: a 3-D map over this call's stack
@@ -901,10 +887,8 @@ int align_chunk_half(mra_handle *h, const float *imgs, int64_t cnt, mra_pose_t *
   t.wait_limit = kWaitLimit;
   t.first_wait_limit = first_wait_limit();
   int rec = prof_begin(h, MRA_STAGE_CC, st);
-  if (h->umma) {
-    t.B16 = static_cast<const uint2 *>(h->B16u);
-    rc = check_launch(h, mra::launch_cc_umma256(&h->tmA, &h->tmB, h->g, t, h->fp16, st),
-                      "tcgen05 contraction/IFFT kernel");
+  if (h->g.hyb_w) {
+    rc = check_launch(h, mra::launch_cc_hybrid256(h->g, t, h->fp16, st), "tcgen05 contraction/IFFT kernel");
   } else {
     rc = check_launch(h, mra::launch_cc_tc(h->g, t, h->fp16, st), "tensor-core contraction/IFFT kernel");
   }
@@ -1044,28 +1028,10 @@ int mra_set_refs(mra_t h, const float *d_refs, int32_t K, mra_stream_t stream) {
   cudaError_t e = cudaMemsetAsync(h->B, 0, static_cast<size_t>(Kpad) * h->NB * sizeof(float2), st);
   if (e != cudaSuccess) return cuda_err(h, e, "cudaMemsetAsync(reference spectra)");
   if (int rc = run_polar(h, d_refs, K, 1, false, true, h->B, nullptr, nullptr, st)) return rc;
-  if (h->umma) {
-    const int ktiles = Kpad / mra::kUmmaRefs;
-    if (!h->B16u || Kpad > h->B16u_refs) {
-      dev_free(h, h->B16u, static_cast<size_t>(h->B16u_refs / mra::kUmmaRefs) * h->g.NU * 2048);
-      h->B16u = nullptr;
-      h->B16u_refs = 0;
-      if (int rc = dev_alloc(h, &h->B16u, static_cast<size_t>(ktiles) * h->g.NU * 2048, "reference k-step tiles"))
-        return rc;
-      h->B16u_refs = Kpad;
-      if (int rc = make_tile_map(h, &h->tmB, h->B16u, static_cast<uint64_t>(ktiles) * h->g.NU * 8, 8 * mra::kUmmaUPerStage,
-                                 "reference k-step tiles"))
-        return rc;
-    }
-    const int rec = prof_begin(h, MRA_STAGE_CONVERT, st);
-    const int rc = check_launch(h, mra::launch_refs16u(h->g, h->B, ktiles, h->B16u, h->fp16, st),
-                                "reference k-step tile kernel");
-    prof_end(h, rec, 1, st);
-    if (rc) return rc;
-  } else if (h->half) {
-    const size_t b16 = static_cast<size_t>(Kpad / mra::kTile) * 2 * h->g.KS * 32 * sizeof(uint2);
+  if (h->half) {
+    const size_t b16 = static_cast<size_t>(Kpad / mra::kTile) * h->g.KS * 32 * sizeof(uint4);
     if (!h->B16 || Kpad > h->B16_refs) {
-      dev_free(h, h->B16, static_cast<size_t>(h->B16_refs / mra::kTile) * 2 * h->g.KS * 32 * sizeof(uint2));
+      dev_free(h, h->B16, static_cast<size_t>(h->B16_refs / mra::kTile) * h->g.KS * 32 * sizeof(uint4));
       h->B16 = nullptr;
       h->B16_refs = 0;
       if (int rc = dev_alloc(h, &h->B16, b16, "reference fragments")) return rc;
@@ -1087,9 +1053,10 @@ int mra_copy_refs(mra_t dst, mra_t src, mra_stream_t stream) {
   if (src == dst) return MRA_OK;
   if (src->K == 0) return set_err(dst, MRA_ESTATE, "source handle holds no references");
   const mra_config_t &a = dst->cfg, &b = src->cfg;
+  auto tcgen05 = [](mra_t h) { return h->half && h->g.M == 256 && h->cfg.kernel == MRA_KERNEL_TCGEN05; };
   if (a.L != b.L || a.first_ring != b.first_ring || a.last_ring != b.last_ring || a.ring_step != b.ring_step ||
       a.shift_range != b.shift_range || a.shift_step != b.shift_step || a.mirror != b.mirror ||
-      a.precision != b.precision || dst->umma != src->umma)
+      a.precision != b.precision || tcgen05(dst) != tcgen05(src))
     return set_err(dst, MRA_EINVAL,
                    "source and destination configurations differ (chunk_images may differ, the kernel may not)");
   if (src->device != dst->device) return set_err(dst, MRA_EINVAL, "source handle lives on another device");
@@ -1109,33 +1076,23 @@ int mra_copy_refs(mra_t dst, mra_t src, mra_stream_t stream) {
   cudaError_t e = cudaMemcpyAsync(dst->B, src->B, static_cast<size_t>(Kpad) * dst->NB * sizeof(float2),
                                   cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return cuda_err(dst, e, "cudaMemcpyAsync(reference spectra)");
-  if (dst->umma) {
-    const int ktiles = Kpad / mra::kUmmaRefs;
-    if (!dst->B16u || Kpad > dst->B16u_refs) {
-      dev_free(dst, dst->B16u, static_cast<size_t>(dst->B16u_refs / mra::kUmmaRefs) * dst->g.NU * 2048);
-      dst->B16u = nullptr;
-      dst->B16u_refs = 0;
-      if (int rc = dev_alloc(dst, &dst->B16u, static_cast<size_t>(ktiles) * dst->g.NU * 2048, "reference k-step tiles"))
-        return rc;
-      dst->B16u_refs = Kpad;
-      if (int rc = make_tile_map(dst, &dst->tmB, dst->B16u, static_cast<uint64_t>(ktiles) * dst->g.NU * 8, 8 * mra::kUmmaUPerStage,
-                                 "reference k-step tiles"))
-        return rc;
-    }
-    e = cudaMemcpyAsync(dst->B16u, src->B16u, static_cast<size_t>(ktiles) * dst->g.NU * 2048,
-                        cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_err(dst, e, "cudaMemcpyAsync(reference k-step tiles)");
-  } else if (dst->half) {
-    const size_t b16 = static_cast<size_t>(Kpad / mra::kTile) * 2 * dst->g.KS * 32 * sizeof(uint2);
+  if (dst->half) {
+    const size_t b16 = static_cast<size_t>(Kpad / mra::kTile) * dst->g.KS * 32 * sizeof(uint4);
     if (!dst->B16 || Kpad > dst->B16_refs) {
-      dev_free(dst, dst->B16, static_cast<size_t>(dst->B16_refs / mra::kTile) * 2 * dst->g.KS * 32 * sizeof(uint2));
+      dev_free(dst, dst->B16, static_cast<size_t>(dst->B16_refs / mra::kTile) * dst->g.KS * 32 * sizeof(uint4));
       dst->B16 = nullptr;
       dst->B16_refs = 0;
       if (int rc = dev_alloc(dst, &dst->B16, b16, "reference fragments")) return rc;
       dst->B16_refs = Kpad;
     }
-    e = cudaMemcpyAsync(dst->B16, src->B16, b16, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_err(dst, e, "cudaMemcpyAsync(reference fragments)");
+    if ((dst->g.hyb_w != nullptr) == (src->g.hyb_w != nullptr)) {
+      e = cudaMemcpyAsync(dst->B16, src->B16, b16, cudaMemcpyDeviceToDevice, st);
+      if (e != cudaSuccess) return cuda_err(dst, e, "cudaMemcpyAsync(reference fragments)");
+    } else {  // the kernels order the k-steps differently: the same values from the FP32 spectra
+      const int rc = check_launch(dst, mra::launch_refs16(dst->g, dst->B, Kpad / mra::kTile, dst->B16, dst->fp16, st),
+                                  "reference fragment kernel");
+      if (rc) return rc;
+    }
   }
   dst->K = src->K;
   return MRA_OK;
