@@ -6,8 +6,7 @@
 namespace mra {
 
 cudaError_t launch_polar16(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
-  if (a.fp16) return g.taps ? launch_polar_t<true, kOutF16>(g, a, st) : launch_polar_t<false, kOutF16>(g, a, st);
-  return g.taps ? launch_polar_t<true, kOutBF16>(g, a, st) : launch_polar_t<false, kOutBF16>(g, a, st);
+  return a.fp16 ? launch_polar_out<kOutF16>(g, a, st) : launch_polar_out<kOutBF16>(g, a, st);
 }
 
 }  // namespace mra

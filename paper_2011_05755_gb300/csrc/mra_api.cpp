@@ -253,13 +253,15 @@ static int fits_shared_memory(const mra_config_t &c, char *why, size_t why_len) 
     const float v = static_cast<float>(-double(c.shift_range) + i * double(c.shift_step));  // as build_tables
     integral = integral && v == std::floor(v);
   }
+  g.NSb = g.NS;
   g.pad = 8;
+  g.pitch = c.L + 16;
   const bool half = c.precision != MRA_FP32;
   struct Need {
     const char *kernel;
     size_t bytes;
   };
-  const Need needs[2] = {{"polar resampling / ring FFT", polar_smem_one_row(g, integral, half)},
+  const Need needs[2] = {{"polar resampling / ring FFT", polar_smem_one_row(g, integral ? kPolarInt : kPolarBare, half)},
                          half ? Need{"FP32 rescore", rescore_smem(g)} : Need{"FP32 contraction", cc_fp32_smem(M, seg_max)}};
   for (const Need &n : needs)
     if (n.bytes > kMaxSmemPerBlock) {
@@ -431,10 +433,11 @@ int build_tables(mra_handle *h) {
     mra::Geometry gp{};
     gp.L = c.L;
     gp.M = M;
-    gp.NS = NS;
+    gp.NSb = NS;
     gp.pad = 8;
+    gp.pitch = c.L + 16;
     gp.KS = mra::kHyb256N0 + 16 * (pattern == 0 ? 13 : 18);
-    if (n3 > 2 || mra::polar_smem_one_row(gp, true, true) > mra::kMaxSmemPerBlock) {
+    if (n3 > 2 || mra::polar_smem_one_row(gp, mra::kPolarInt, true) > mra::kMaxSmemPerBlock) {
       pattern = -1;
     } else {
       std::vector<int2> info;
@@ -490,44 +493,6 @@ int build_tables(mra_handle *h) {
       shifts[iy * nx + ix] = make_float2(static_cast<float>(-double(c.shift_range) + ix * double(c.shift_step)),
                                          static_cast<float>(-double(c.shift_range) + iy * double(c.shift_step)));
 
-  // Taps for integer shift grids (the sample position c0 + o in FP32, as the
-  // kernel would form it; an integer shift moves only the tap index).
-  std::vector<float4> taps;
-  int pad = -1;
-  {
-    bool integral = true;
-    for (const float2 &sv : shifts) integral = integral && sv.x == std::floor(sv.x) && sv.y == std::floor(sv.y);
-    int smax = 0;
-    for (const float2 &sv : shifts)
-      smax = std::max(smax, static_cast<int>(std::max(std::fabs(sv.x), std::fabs(sv.y))));
-    if (integral) {
-      const float c0 = 0.5f * static_cast<float>(c.L);
-      int lo = 0, hi = 0;
-      std::vector<int2> base(NS);
-      std::vector<float2> frac(NS);
-      for (int q = 0; q < NS; ++q) {
-        const float x = c0 + offs[q].x, y = c0 + offs[q].y;
-        const float xf = std::floor(x), yf = std::floor(y);
-        base[q] = make_int2(static_cast<int>(xf), static_cast<int>(yf));
-        frac[q] = make_float2(x - xf, y - yf);
-        lo = std::min(lo, std::min(base[q].x, base[q].y) - smax);
-        hi = std::max(hi, std::max(base[q].x, base[q].y) + 1 + smax - (c.L - 1));
-      }
-      const int need = std::max(-lo, hi);
-      if (need <= 8) {
-        pad = need <= 4 ? 4 : 8;  // a multiple of 4 keeps the interior float4-aligned
-        const int Lp = c.L + 2 * pad;
-        taps.resize(NS);
-        for (int q = 0; q < NS; ++q) {
-          const int idx = (base[q].y + pad) * Lp + (base[q].x + pad);
-          float fidx;
-          std::memcpy(&fidx, &idx, 4);
-          taps[q] = make_float4(fidx, frac[q].x, frac[q].y, 0.f);
-        }
-      }
-    }
-  }
-
   mra::Geometry &g = h->g;
   g.L = c.L;
   g.M = M;
@@ -542,11 +507,6 @@ int build_tables(mra_handle *h) {
   int rc;
   if ((rc = upload(h, offs, &g.offs, "ring offsets"))) return rc;
   g.taps = nullptr;
-  g.pad = 0;
-  if (pad >= 0) {
-    if ((rc = upload(h, taps, &g.taps, "bilinear taps"))) return rc;
-    g.pad = pad;
-  }
   if ((rc = upload(h, rings, &g.rings, "ring table"))) return rc;
   if ((rc = upload(h, binpos, &g.binpos, "bin positions"))) return rc;
   if ((rc = upload(h, bweight, &g.bweight, "ring weights"))) return rc;
@@ -556,6 +516,85 @@ int build_tables(mra_handle *h) {
   if ((rc = upload(h, ang, &g.angles, "angle table"))) return rc;
   if ((rc = upload(h, fseg, &g.fseg, "frequency segments"))) return rc;
   g.KS = static_cast<int>(ksinfo.size());
+  // Polar kernel: the image inside a zero border that every neighbour of every
+  // sample stays in, where the border needs at most 8 pixels (the sample
+  // position c0 + s + o in FP32, as the kernel forms it; an integer shift
+  // moves only the tap index).
+  {
+    bool integral = true;
+    for (const float2 &sv : shifts) integral = integral && sv.x == std::floor(sv.x) && sv.y == std::floor(sv.y);
+    int smax = 0;
+    for (const float2 &sv : shifts)
+      smax = std::max(smax, static_cast<int>(std::ceil(std::max(std::fabs(sv.x), std::fabs(sv.y)))));
+    const float c0 = 0.5f * static_cast<float>(c.L);
+    int lo = 0, hi = 0;
+    for (int q = 0; q < NS; ++q) {
+      const int bx = static_cast<int>(std::floor(c0 + offs[q].x)), by = static_cast<int>(std::floor(c0 + offs[q].y));
+      lo = std::min(lo, std::min(bx, by) - smax);
+      hi = std::max(hi, std::max(bx, by) + 1 + smax - (c.L - 1));
+    }
+    if (!integral) {  // the rounded sum may fall a pixel either side of the rounded parts
+      --lo;
+      ++hi;
+    }
+    const int need = std::max(-lo, hi);
+    g.mode = mra::kPolarBare;
+    g.NSb = NS;
+    g.pad = g.pitch = 0;
+    const int out16 = h->half;
+    const int bare_rows = mra::polar_rows_per_cta(g, mra::kPolarBare, out16);
+    if (need <= 8) {
+      mra::Geometry t = g;
+      const int mode = integral ? mra::kPolarInt : mra::kPolarFrac;
+      t.pad = need <= 4 ? 4 : 8;  // a multiple of 4 keeps the interior float4-aligned
+      t.pitch = c.L + 2 * t.pad;
+      // a fractional grid takes the border only where it costs no row of the CTA
+      const bool fits = integral || (mra::polar_smem_one_row(t, mode, out16) <= mra::kMaxSmemPerBlock &&
+                                     mra::polar_rows_per_cta(t, mode, out16) == bare_rows);
+      if (fits) {
+        g = t;
+        g.mode = mode;
+        // rows a multiple of 16 floats long (or nearly) put vertical neighbours in the same banks
+        // (4.3 to 5.5 wavefronts per read at pitch 0 mod 32, 2.8 at 2, 16 and 30, about 2 elsewhere),
+        // and rings of one length start in the same bank: both are mended where there is room for it
+        t = g;
+        while (t.pitch % 32 == 0 || t.pitch % 32 == 2 || t.pitch % 32 == 16 || t.pitch % 32 == 30) t.pitch += 4;
+        t.NSb = NS + 8 * NR;
+        if (t.pitch <= 256 && t.NSb < 65536 && mra::polar_smem_one_row(t, mode, out16) <= mra::kMaxSmemPerBlock &&
+            mra::polar_rows_per_cta(t, mode, out16) == mra::polar_rows_per_cta(g, mode, out16))
+          g = t;
+      }
+    }
+    std::vector<int4> prings = rings;
+    if (g.NSb > NS)
+      for (int i = 0; i < NR; ++i) prings[i].y += 8 * i;
+    if ((rc = upload(h, prings, &g.prings, "ring table of the sample buffer"))) return rc;
+    if (g.mode != mra::kPolarBare) {
+      // samples in patches of up to 5 rings of one length x 8 angles
+      std::vector<float4> taps;
+      taps.reserve(NS);
+      for (int i0 = 0, i1; i0 < NR; i0 = i1) {
+        for (i1 = i0 + 1; i1 < NR && i1 < i0 + 5 && NN[i1] == NN[i0];) ++i1;
+        for (int q0 = 0; q0 < NN[i0]; q0 += 8)
+          for (int i = i0; i < i1; ++i)
+            for (int k = q0; k < q0 + 8 && k < NN[i]; ++k) {
+              const int q = rings[i].y + k, at = (prings[i].y + k) | q << 16;
+              float fat, fidx;
+              std::memcpy(&fat, &at, 4);
+              if (g.mode == mra::kPolarFrac) {
+                taps.push_back(make_float4(fat, offs[q].x, offs[q].y, 0.f));
+                continue;
+              }
+              const float x = c0 + offs[q].x, y = c0 + offs[q].y;
+              const float xf = std::floor(x), yf = std::floor(y);
+              const int idx = (static_cast<int>(yf) + g.pad) * g.pitch + static_cast<int>(xf) + g.pad;
+              std::memcpy(&fidx, &idx, 4);
+              taps.push_back(make_float4(fidx, x - xf, y - yf, fat));
+            }
+      }
+      if ((rc = upload(h, taps, &g.taps, "sample table"))) return rc;
+    }
+  }
   if ((rc = upload(h, kso, &g.kso, "k-step offsets"))) return rc;
   if ((rc = upload(h, ksinfo, &g.ksinfo, "k-step table"))) return rc;
   if ((rc = upload(h, binpos16, &g.binpos16, "16-bit bin positions"))) return rc;
@@ -851,13 +890,13 @@ int run_polar(mra_handle *h, const float *imgs, int64_t n, int rows_per_img, boo
   // (rows of L * 4 bytes must be a multiple of 16, the base 16-byte
   // aligned, the bordered box at most 256 wide); else plain loads
   {
-    const int L = h->g.L, pad = h->g.taps ? h->g.pad : 0, Lp = L + 2 * pad;
-    const TensorMapEncode encode = (L % 4 == 0 && Lp <= 256 && (reinterpret_cast<uintptr_t>(imgs) & 15) == 0)
+    const int L = h->g.L, pad = h->g.pad, Lp = L + 2 * pad, W = pad ? h->g.pitch : L;
+    const TensorMapEncode encode = (L % 4 == 0 && W <= 256 && (reinterpret_cast<uintptr_t>(imgs) & 15) == 0)
                                        ? tensor_map_encoder() : nullptr;
     if (encode) {
       const cuuint64_t dims[3] = {static_cast<cuuint64_t>(L), static_cast<cuuint64_t>(L), static_cast<cuuint64_t>(n)};
       const cuuint64_t strides[2] = {static_cast<cuuint64_t>(L) * 4, static_cast<cuuint64_t>(L) * L * 4};
-      const cuuint32_t box[3] = {static_cast<cuuint32_t>(Lp), static_cast<cuuint32_t>(Lp), 1};
+      const cuuint32_t box[3] = {static_cast<cuuint32_t>(W), static_cast<cuuint32_t>(Lp), 1};
       const cuuint32_t estr[3] = {1, 1, 1};
       a.tma = encode(&a.tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(imgs), dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -15,6 +15,8 @@ namespace mra {
 // bin are contiguous (float2 each), so one bin of a tile is 64 bytes.
 constexpr int kTile = 8;
 
+enum PolarMode { kPolarBare = 0, kPolarInt = 1, kPolarFrac = 2 };
+
 // Geometry tables on the device (built in FP64 on the host, stored FP32).
 struct Geometry {
   int L;            // box size
@@ -26,12 +28,16 @@ struct Geometry {
   int S;            // shifts
   int mirror;       // 0/1
   const float2 *offs;     // [NS]  r (cos theta_q, sin theta_q)
-  // Integer shift grids: bilinear taps of the unshifted sample positions in
-  // a copy of the image with a zero border of `pad` pixels (row length
-  // L + 2 pad); tap q = {index of the top-left neighbour (int bits), fx, fy}.
-  // Null when the shift grid is not integer or the border would exceed 8.
-  const float4 *taps;     // [NS] or null
-  int pad;
+  // Polar kernel (PolarMode): where the image fits shared memory inside a zero
+  // border of `pad` (4 or 8) pixels, rows of `pitch` floats, a table of the
+  // samples in the order they are taken.  kPolarInt: {index of the top-left
+  // neighbour of the unshifted position (int bits), fx, fy, place (int bits)};
+  // kPolarFrac: {place, offset x, offset y, -}; place = offset in the sample
+  // buffer | number in ring order << 16.
+  const float4 *taps;     // [NS], null for kPolarBare
+  int mode, pad, pitch;
+  const int4 *prings;     // [NR] the ring table with offsets into the sample buffer of NSb floats
+  int NSb;
   const int4 *rings;      // [NR]  {N_r, sample offset, natural-bin offset, log2(N_r/2)}
   const int *binpos;      // [NBIN] padded position of (ring, f), ring-major natural order
   const float *bweight;   // [NBIN] reference-side weight of (ring, f)
@@ -140,7 +146,8 @@ size_t rescore_smem(const Geometry &g);
 int rescore_ctas_per_sm(const Geometry &g);  // resident rescore CTAs per SM (0 if unknown)
 // Shared memory of one CTA of the polar kernel with one row, of the FP32
 // contraction kernel, and the per-CTA opt-in limit of the device.
-size_t polar_smem_one_row(const Geometry &g, bool taps, bool out16);
+size_t polar_smem_one_row(const Geometry &g, int mode, bool out16);
+int polar_rows_per_cta(const Geometry &g, int mode, bool out16);
 size_t cc_fp32_smem(int M, int seg_max);
 constexpr size_t kMaxSmemPerBlock = 232448;  // 227 KB
 // Every check mra_create makes on a configuration, without CUDA calls or heap

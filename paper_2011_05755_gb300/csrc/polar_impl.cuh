@@ -29,10 +29,10 @@
 
 namespace mra {
 
-// Row stride of the sample buffer: >= NS and 16 floats off a multiple of 32,
-// so the ring-FFT jobs of consecutive rows start in opposite halves of the
-// shared-memory banks.
-__host__ __device__ inline int sample_stride(int NS) { return NS + ((16 - NS) & 31); }
+// Row stride of the sample buffer (NSb floats a row): 16 floats off a
+// multiple of 32, so the ring-FFT jobs of consecutive rows start in opposite
+// halves of the shared-memory banks.
+__host__ __device__ inline int sample_stride(int NSb) { return NSb + ((16 - NSb) & 31); }
 
 // Output layouts of the polar kernel: FP32 frequency-major tiles, or the
 // 16-bit q / p planes (BF16 or FP16) that phase 3 turns into mma.sync
@@ -63,12 +63,12 @@ __device__ __forceinline__ int plane_swz(int w) { return w ^ ((w >> 4) & 14); }
 template <int OUT>
 __device__ __forceinline__ void put_bin(const Geometry &g, const PolarArgs &a, uint32_t *planes_row, const int *s_kpos,
                                         int ring, int bin0, int64_t row, int k, float2 X) {
-  if (a.weighted) {
+  if (OUT == kOutF32 && a.weighted) {  // references and debug copies take the FP32 output
     const float w = g.bweight[bin0 + k];
     X.x *= w;
     X.y *= w;
   }
-  if (a.dbg_spec) a.dbg_spec[row * g.NBIN + bin0 + k] = X;
+  if (OUT == kOutF32 && a.dbg_spec) a.dbg_spec[row * g.NBIN + bin0 + k] = X;
   if constexpr (OUT == kOutF32) {
     if (a.out) a.out[((row >> 3) * g.NB + s_kpos[k] + ring) * kTile + (row & 7)] = X;
   } else {
@@ -99,8 +99,8 @@ __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a,
     // (ring, row) of the job; nrows is R except in an image's last group
     const int ring = i0 + (nrows == R ? jc / R : jc / nrows);
     const int i = nrows == R ? jc % R : jc % nrows;
-    const int4 rd = g.rings[ring];  // {N, sample offset, natural-bin offset, log2(N/2)}
-    float2 *z = reinterpret_cast<float2 *>(smem + i * sample_stride(g.NS) + rd.y);
+    const int4 rd = g.prings[ring];  // {N, offset in the sample buffer, natural-bin offset, log2(N/2)}
+    float2 *z = reinterpret_cast<float2 *>(smem + i * sample_stride(g.NSb) + rd.y);
     group_fft<H>(z, t, active, tws, g.M);
     if (active) {
       const int wstep = g.M / (2 * H);
@@ -119,23 +119,26 @@ __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a,
   return (first_warp + (njobs + JPW - 1) / JPW) % nwarps;  // first warp of the next class
 }
 
-// Shared-memory image floats: the image, or (TAPS) the image inside a zero
-// border of g.pad pixels.
-__host__ __device__ inline int image_floats(const Geometry &g, bool taps) {
-  const int Lp = taps ? g.L + 2 * g.pad : g.L;
-  return (Lp * Lp + 3) & ~3;
+// Shared-memory image: the bare image, sampled with bounds checks
+// (kPolarBare), or the image inside a zero border of g.pad pixels with rows
+// of g.pitch floats, where every neighbour of every sample is in the buffer:
+// integer shift grids (kPolarInt), whose bilinear weights do not depend on
+// the shift, and other grids (kPolarFrac).
+__host__ __device__ inline int image_floats(const Geometry &g, int mode) {
+  const int n = mode == kPolarBare ? g.L * g.L : (g.L + 2 * g.pad) * g.pitch;
+  return (n + 3) & ~3;
 }
 
-template <int R, bool TAPS, int OUT>
+template <int R, int MODE, int OUT>
 __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
   extern __shared__ float4 smem_f4[];
   const int L = g.L, NS = g.NS, M = g.M;
-  const int NSp = sample_stride(NS);
+  const int NSp = sample_stride(g.NSb);
   const int LL = L * L;
   const int64_t img = blockIdx.y;
-  float *im = reinterpret_cast<float *>(smem_f4);       // the image (with its zero border if TAPS)
-  uint64_t *ibar = reinterpret_cast<uint64_t *>(im + image_floats(g, TAPS));  // image copy barrier (16 B)
-  float2 *tws = reinterpret_cast<float2 *>(im + image_floats(g, TAPS) + 4);  // [M] forward twiddles
+  float *im = reinterpret_cast<float *>(smem_f4);       // the image (with its zero border unless kPolarBare)
+  uint64_t *ibar = reinterpret_cast<uint64_t *>(im + image_floats(g, MODE));  // image copy barrier (16 B)
+  float2 *tws = reinterpret_cast<float2 *>(im + image_floats(g, MODE) + 4);  // [M] forward twiddles
   int *s_kpos = reinterpret_cast<int *>(tws + M);       // [M/2 + 1] output bases (padded to even)
   float *smem = reinterpret_cast<float *>(s_kpos + ((M / 2 + 2) & ~1));  // [R][NSp] samples, then ring FFTs
   const float c0 = 0.5f * static_cast<float>(L);
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
   }
   const float *src = a.imgs + img * LL;
   const bool vec = (L & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-  // TMA staging: one tensor copy of the image (and, with TAPS, its zero
+  // TMA staging: one tensor copy of the image (and, where it has one, its zero
   // border from the map's out-of-bounds fill), issued by thread 0 while the
   // CTA loads its tables; the destination must be 128-byte aligned
   const bool tma = a.tma && (smem_u32(im) & 127u) == 0;
@@ -159,15 +162,14 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
     if (threadIdx.x == 0) {
       mbar_init(ibar, 1);
       mbar_init_fence();
-      const int pad = TAPS ? g.pad : 0;
-      const int Lp = L + 2 * pad;
-      mbar_arrive_expect_tx(ibar, static_cast<uint32_t>(Lp * Lp) * 4u);
+      const int pad = MODE ? g.pad : 0;
+      mbar_arrive_expect_tx(ibar, static_cast<uint32_t>(MODE ? (L + 2 * pad) * g.pitch : LL) * 4u);
       tma_load_3d(im, &a.tmap, -pad, -pad, static_cast<int>(img), ibar);
     }
-  } else if constexpr (TAPS) {
+  } else if constexpr (MODE != kPolarBare) {
     // zero the bordered buffer, then copy the interior (pad is a multiple of 4)
-    const int Lp = L + 2 * g.pad;
-    for (int i = threadIdx.x; i < image_floats(g, true) / 4; i += blockDim.x)
+    const int Lp = g.pitch;
+    for (int i = threadIdx.x; i < image_floats(g, MODE) / 4; i += blockDim.x)
       reinterpret_cast<float4 *>(im)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     float *dst = im + g.pad * Lp + g.pad;
@@ -209,11 +211,17 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
     const int nrows = min(R, a.rows_per_img - s0);
     const int64_t row0 = img * a.rows_per_img + s0;
     // Phase 1: samples x_r(theta_q) = I(c0 + s + r (cos theta_q, sin theta_q)).
-    if constexpr (TAPS) {
+    // The table lists the samples in patches of up to 5 adjacent rings x 8
+    // angles, which spread the reads of a warp over the banks better than 32
+    // samples along one ring (1.8 to 2.0 wavefronts per read against 2.4 to
+    // 2.8, counted over the table's batches), with each sample's place in the
+    // buffer (low 16 bits) and its number in ring order (high 16 bits).
+    if constexpr (MODE == kPolarInt) {
       // integer shifts: the bilinear weights of a sample do not depend on the
       // shift, which only moves the neighbourhood inside the bordered image
-      const int Lp = L + 2 * g.pad;
+      const int Lp = g.pitch;
       int soff[R];
+      bool run = nrows == R;  // the group's shifts step along x by one pixel
 #pragma unroll
       for (int i = 0; i < R; ++i) {
         soff[i] = 0;
@@ -221,6 +229,7 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
           const float2 sh = g.shifts[s0 + i];
           soff[i] = static_cast<int>(sh.y) * Lp + static_cast<int>(sh.x);
         }
+        if (i > 0) run = run && soff[i] == soff[i - 1] + 1;
       }
       // eight samples per thread and pass, their tap loads issued together
       constexpr int QU = 8;
@@ -235,15 +244,31 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
         for (int u = 0; u < QU; ++u) {
           const int q = q0 + u * blockDim.x;
           if (q < NS) {
-            const int base = __float_as_int(tp[u].x);
+            const int at = __float_as_int(tp[u].w);
             const float fx = tp[u].y, fy = tp[u].z, gx = 1.f - fx, gy = 1.f - fy;
+            const float *p = im + __float_as_int(tp[u].x) + soff[0];
+            float *dst = smem + (at & 0xffff);
+            auto put = [&](int i, float v) {
+              dst[i * NSp] = v;
+              if (OUT == kOutF32 && a.dbg_samples) a.dbg_samples[(row0 + i) * NS + (at >> 16)] = v;
+            };
+            if (R > 1 && run) {  // neighbouring rows share the pixel columns between them
+              float t[R + 1], b[R + 1];
 #pragma unroll
-            for (int i = 0; i < R; ++i) {
-              if (i < nrows) {
-                const float *p = im + base + soff[i];
-                const float v = gy * (gx * p[0] + fx * p[1]) + fy * (gx * p[Lp] + fx * p[Lp + 1]);
-                smem[i * NSp + q] = v;
-                if (a.dbg_samples) a.dbg_samples[(row0 + i) * NS + q] = v;
+              for (int i = 0; i <= R; ++i) {
+                t[i] = p[i];
+                b[i] = p[Lp + i];
+              }
+#pragma unroll
+              for (int i = 0; i < R; ++i)
+                put(i, gy * (gx * t[i] + fx * t[i + 1]) + fy * (gx * b[i] + fx * b[i + 1]));
+            } else {
+#pragma unroll
+              for (int i = 0; i < R; ++i) {
+                if (i < nrows) {
+                  const float *pi = p + (soff[i] - soff[0]);
+                  put(i, gy * (gx * pi[0] + fx * pi[1]) + fy * (gx * pi[Lp] + fx * pi[Lp + 1]));
+                }
               }
             }
           }
@@ -261,14 +286,36 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
           cy[i] += sh.y;
         }
       }
-      for (int q = threadIdx.x; q < NS; q += blockDim.x) {
-        const float2 o = g.offs[q];
+      if constexpr (MODE == kPolarFrac) {
+        const int Lp = g.pitch;
+        const float *im0 = im + g.pad * Lp + g.pad;  // pixel (0, 0)
+#pragma unroll 4
+        for (int q = threadIdx.x; q < NS; q += blockDim.x) {
+          const float4 tp = __ldg(g.taps + q);  // {place, offset x, offset y}
+          const int at = __float_as_int(tp.x);
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-          if (i < nrows) {
-            const float v = bilinear_smem(im, L, cx[i] + o.x, cy[i] + o.y);
-            smem[i * NSp + q] = v;
-            if (a.dbg_samples) a.dbg_samples[(row0 + i) * NS + q] = v;
+          for (int i = 0; i < R; ++i) {
+            if (i < nrows) {
+              const float x = cx[i] + tp.y, y = cy[i] + tp.z;
+              const float xf = floorf(x), yf = floorf(y);
+              const float fx = x - xf, fy = y - yf, gx = 1.f - fx, gy = 1.f - fy;
+              const float *p = im0 + static_cast<int>(yf) * Lp + static_cast<int>(xf);
+              const float v = gy * (gx * p[0] + fx * p[1]) + fy * (gx * p[Lp] + fx * p[Lp + 1]);
+              smem[i * NSp + (at & 0xffff)] = v;
+              if (OUT == kOutF32 && a.dbg_samples) a.dbg_samples[(row0 + i) * NS + (at >> 16)] = v;
+            }
+          }
+        }
+      } else {
+        for (int q = threadIdx.x; q < NS; q += blockDim.x) {
+          const float2 o = g.offs[q];  // the bare mode's buffer is in ring order
+#pragma unroll
+          for (int i = 0; i < R; ++i) {
+            if (i < nrows) {
+              const float v = bilinear_smem(im, L, cx[i] + o.x, cy[i] + o.y);
+              smem[i * NSp + q] = v;
+              if (OUT == kOutF32 && a.dbg_samples) a.dbg_samples[(row0 + i) * NS + q] = v;
+            }
           }
         }
       }
@@ -327,10 +374,10 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
   }
 }
 
-template <int R, bool TAPS, int OUT>
+template <int R, int MODE, int OUT>
 static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t smem, cudaStream_t st) {
   static size_t granted = 0;
-  cudaError_t e = raise_smem_limit(polar_fft_kernel<R, TAPS, OUT>, smem, granted);
+  cudaError_t e = raise_smem_limit(polar_fft_kernel<R, MODE, OUT>, smem, granted);
   if (e != cudaSuccess) return e;
   // CTAs per image (each walks its share of the image's shift groups and
   // stages the image once): four when two or more CTAs fit on an SM, so
@@ -353,36 +400,50 @@ static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t 
   if (per_img < want) per_img = want;
   if (per_img > groups) per_img = groups;
   dim3 grid(static_cast<unsigned>(per_img), static_cast<unsigned>(a.n_imgs));
-  polar_fft_kernel<R, TAPS, OUT><<<grid, 256, smem, st>>>(g, a);
+  polar_fft_kernel<R, MODE, OUT><<<grid, 256, smem, st>>>(g, a);
   return cudaGetLastError();
 }
 
 // Shared memory of a CTA with R rows: the staged image, its copy barrier,
 // the twiddles, the output bases, then per row the samples and (16-bit
 // output) the planes.
-inline size_t polar_smem_bytes(const Geometry &g, bool taps, bool out16, int R) {
-  const size_t fixed = static_cast<size_t>(image_floats(g, taps)) * sizeof(float) + 16 + g.M * sizeof(float2) +
+inline size_t polar_smem_bytes(const Geometry &g, int mode, bool out16, int R) {
+  const size_t fixed = static_cast<size_t>(image_floats(g, mode)) * sizeof(float) + 16 + g.M * sizeof(float2) +
                        static_cast<size_t>((g.M / 2 + 2) & ~1) * sizeof(int);
-  size_t per_row = static_cast<size_t>(sample_stride(g.NS)) * sizeof(float);
+  size_t per_row = static_cast<size_t>(sample_stride(g.NSb)) * sizeof(float);
   if (out16) per_row += static_cast<size_t>(g.KS) * 16 * sizeof(uint32_t);
   return fixed + per_row * R;
 }
 
-template <bool TAPS, int OUT>
-static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
-  const size_t fixed = polar_smem_bytes(g, TAPS, OUT != kOutF32, 0);
-  const size_t per_row = polar_smem_bytes(g, TAPS, OUT != kOutF32, 1) - fixed;
-  // two CTAs per SM when the rows fit in ~110 KB, else as many rows as fit in 200 KB
+// Rows (shifts) per CTA: as many as let two CTAs fit on an SM (~110 KB), else
+// as many as fit in 200 KB.
+inline int polar_cta_rows(const Geometry &g, int mode, bool out16) {
+  const size_t fixed = polar_smem_bytes(g, mode, out16, 0);
+  const size_t per_row = polar_smem_bytes(g, mode, out16, 1) - fixed;
   int R = static_cast<int>((112640 > fixed ? 112640 - fixed : 0) / per_row);
   if (R < 1) R = static_cast<int>((204800 > fixed ? 204800 - fixed : 0) / per_row);
-  R = R < 1 ? 1 : (R > 4 ? 4 : R);
+  return R < 1 ? 1 : (R > 4 ? 4 : R);
+}
+
+template <int MODE, int OUT>
+static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
+  int R = polar_cta_rows(g, MODE, OUT != kOutF32);
   if (R > a.rows_per_img) R = a.rows_per_img;
-  const size_t smem = fixed + per_row * R;
+  const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
   switch (R) {
-    case 1: return launch_polar_r<1, TAPS, OUT>(g, a, smem, st);
-    case 2: return launch_polar_r<2, TAPS, OUT>(g, a, smem, st);
-    case 3: return launch_polar_r<3, TAPS, OUT>(g, a, smem, st);
-    default: return launch_polar_r<4, TAPS, OUT>(g, a, smem, st);
+    case 1: return launch_polar_r<1, MODE, OUT>(g, a, smem, st);
+    case 2: return launch_polar_r<2, MODE, OUT>(g, a, smem, st);
+    case 3: return launch_polar_r<3, MODE, OUT>(g, a, smem, st);
+    default: return launch_polar_r<4, MODE, OUT>(g, a, smem, st);
+  }
+}
+
+template <int OUT>
+static cudaError_t launch_polar_out(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
+  switch (g.mode) {
+    case kPolarInt: return launch_polar_t<kPolarInt, OUT>(g, a, st);
+    case kPolarFrac: return launch_polar_t<kPolarFrac, OUT>(g, a, st);
+    default: return launch_polar_t<kPolarBare, OUT>(g, a, st);
   }
 }
 
