@@ -6,7 +6,7 @@
 namespace mra {
 
 cudaError_t launch_polar16(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
-  return a.fp16 ? launch_polar_out<kOutF16>(g, a, st) : launch_polar_out<kOutBF16>(g, a, st);
+  return launch_polar_out<kOut16>(g, a, st);
 }
 
 }  // namespace mra

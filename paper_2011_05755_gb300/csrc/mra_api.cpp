@@ -565,10 +565,11 @@ int build_tables(mra_handle *h) {
           g = t;
       }
     }
-    std::vector<int4> prings = rings;
-    if (g.NSb > NS)
-      for (int i = 0; i < NR; ++i) prings[i].y += 8 * i;
-    if ((rc = upload(h, prings, &g.prings, "ring table of the sample buffer"))) return rc;
+    g.nx = nx;
+    g.smin = static_cast<int>(shifts[0].x);
+    g.sstep = nx > 1 ? static_cast<int>(shifts[1].x) - g.smin : 1;
+    const int gap = g.NSb > NS ? 8 : 0;
+    mra::set_ring_classes(g, rings.data(), NR, gap);
     if (g.mode != mra::kPolarBare) {
       // samples in patches of up to 5 rings of one length x 8 angles
       std::vector<float4> taps;
@@ -578,7 +579,7 @@ int build_tables(mra_handle *h) {
         for (int q0 = 0; q0 < NN[i0]; q0 += 8)
           for (int i = i0; i < i1; ++i)
             for (int k = q0; k < q0 + 8 && k < NN[i]; ++k) {
-              const int q = rings[i].y + k, at = (prings[i].y + k) | q << 16;
+              const int q = rings[i].y + k, at = (rings[i].y + gap * i + k) | q << 16;
               float fat, fidx;
               std::memcpy(&fat, &at, 4);
               if (g.mode == mra::kPolarFrac) {

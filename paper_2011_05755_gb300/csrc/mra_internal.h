@@ -15,6 +15,15 @@ namespace mra {
 // bin are contiguous (float2 each), so one bin of a tile is 64 bytes.
 constexpr int kTile = 8;
 
+// Rings [i0, i1) of one length 2 H: ring i's samples start at float
+// off + (i - i0) stride of a row's sample buffer, its bins at natural-order
+// bin + (i - i0) (H + 1).
+struct RingClass {
+  int i0, i1, H, off, stride, bin;
+};
+
+constexpr int kRingClasses = 7;
+
 enum PolarMode { kPolarBare = 0, kPolarInt = 1, kPolarFrac = 2 };
 
 // Geometry tables on the device (built in FP64 on the host, stored FP32).
@@ -36,8 +45,12 @@ struct Geometry {
   // buffer | number in ring order << 16.
   const float4 *taps;     // [NS], null for kPolarBare
   int mode, pad, pitch;
-  const int4 *prings;     // [NR] the ring table with offsets into the sample buffer of NSb floats
-  int NSb;
+  int nx, smin, sstep;    // kPolarInt: shift s = iy nx + ix is (smin + ix sstep, smin + iy sstep)
+  // rings of length 512, 256, ..., 8 (i0 = i1: none), passed by value: walking
+  // the ring table in memory for the class boundaries was a chain of NR
+  // dependent loads per group of rows (12 % of the kernel)
+  RingClass cls[kRingClasses];
+  int NSb;                // floats of a row's sample buffer
   const int4 *rings;      // [NR]  {N_r, sample offset, natural-bin offset, log2(N_r/2)}
   const int *binpos;      // [NBIN] padded position of (ring, f), ring-major natural order
   const float *bweight;   // [NBIN] reference-side weight of (ring, f)
@@ -153,6 +166,20 @@ constexpr size_t kMaxSmemPerBlock = 232448;  // 227 KB
 // Every check mra_create makes on a configuration, without CUDA calls or heap
 // use: MRA_OK, MRA_EINVAL or MRA_EUNSUPPORTED with a message in why.
 int check_config(const mra_config_t *c, char *why, size_t why_len);
+
+// Ring classes of a geometry with NR rings (ascending lengths), `gap` floats
+// between consecutive rings in the sample buffer; sets cls and NSb.
+inline void set_ring_classes(Geometry &g, const int4 *rings, int NR, int gap) {
+  for (int k = 0; k < kRingClasses; ++k) g.cls[k] = RingClass{0, 0, 256 >> k, 0, 0, 0};
+  for (int i = 0; i < NR; ++i) {
+    const int N = rings[i].x;
+    int k = 0;
+    while (512 >> k > N) ++k;
+    if (g.cls[k].i1 == 0) g.cls[k] = RingClass{i, i, N / 2, rings[i].y + gap * i, N + gap, rings[i].z};
+    g.cls[k].i1 = i + 1;
+  }
+  g.NSb = rings[NR - 1].y + rings[NR - 1].x + gap * NR;
+}
 
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_polar(const Geometry &g, const PolarArgs &a, cudaStream_t st);

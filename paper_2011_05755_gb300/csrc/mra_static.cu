@@ -272,8 +272,7 @@ int mra_align_static(const mra_config_t *cfg, const float *d_refs, int32_t K, co
 #undef MRA_COPY
   g.offs = d_offs;
   g.rings = d_rings;
-  g.prings = d_rings;  // bare mode: the sample buffer is in ring order
-  g.NSb = NS;
+  mra::set_ring_classes(g, h_rings, NR, 0);
   g.binpos = d_binpos;
   g.bweight = d_bweight;
   g.fwd_tw = d_fwd;

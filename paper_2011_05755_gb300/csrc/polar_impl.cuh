@@ -37,18 +37,16 @@ __host__ __device__ inline int sample_stride(int NSb) { return NSb + ((16 - NSb)
 // Output layouts of the polar kernel: FP32 frequency-major tiles, or the
 // 16-bit q / p planes (BF16 or FP16) that phase 3 turns into mma.sync
 // fragments.
-enum PolarOut { kOutF32 = 0, kOutBF16 = 1, kOutF16 = 2 };
+enum PolarOut { kOutF32 = 0, kOut16 = 1 };
 
 // (q, p) of one bin packed as a 16-bit pair word: q low, p high.
-template <int OUT>
-__device__ __forceinline__ uint32_t pack_qp(float q, float p) {
-  if constexpr (OUT == kOutF16) {
+__device__ __forceinline__ uint32_t pack_qp(float q, float p, bool fp16) {
+  if (fp16) {
     const __half2 h = __floats2half2_rn(q, p);  // .x (low half) = q
     return *reinterpret_cast<const uint32_t *>(&h);
-  } else {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(q, p);
-    return *reinterpret_cast<const uint32_t *>(&h);
   }
+  const __nv_bfloat162 h = __floats2bfloat162_rn(q, p);
+  return *reinterpret_cast<const uint32_t *>(&h);
 }
 
 // Position of word w (k-step w / 16, word w % 16) in a row of the (q, p)
@@ -73,22 +71,22 @@ __device__ __forceinline__ void put_bin(const Geometry &g, const PolarArgs &a, u
     if (a.out) a.out[((row >> 3) * g.NB + s_kpos[k] + ring) * kTile + (row & 7)] = X;
   } else {
     const int w = s_kpos[k] + ring;  // k-step w / 16, word w % 16 of it
-    planes_row[plane_swz(w)] = pack_qp<OUT>(X.x - X.y, X.x + X.y);
+    planes_row[plane_swz(w)] = pack_qp(X.x - X.y, X.x + X.y, a.fp16);
   }
 }
 
-// All (ring, row) jobs of one ring-length class [i0, i1) of a CTA: forward
+// All (ring, row) jobs of one ring-length class c of a CTA: forward
 // FFT of the packed samples, real split, weights, and the spectrum written in
 // the layout the path needs (FP32 tiled, 16-bit q/p words, debug).  s_kpos
 // holds the per-frequency base of the output layout: bin (ring, k) goes to
 // s_kpos[k] + ring.
 template <int H, int R, int OUT>
 __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a, float *smem, uint32_t *planes,
-                                          int NB16, const float2 *tws, const int *s_kpos, int i0, int i1, int nrows,
+                                          int NB16, const float2 *tws, const int *s_kpos, const RingClass &c, int nrows,
                                           int64_t row0, int warp, int lane, int nwarps, int first_warp) {
   constexpr int T = GroupFft<H>::T;
   constexpr int JPW = 32 / T;  // jobs per warp pass
-  const int njobs = (i1 - i0) * nrows;
+  const int njobs = (c.i1 - c.i0) * nrows;
   const int t = lane % T;
   // warp passes of this class start after the previous class's last pass
   const int wslot = (warp - first_warp + nwarps) % nwarps;
@@ -97,10 +95,10 @@ __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a,
     const bool active = job < njobs;
     const int jc = active ? job : j0;
     // (ring, row) of the job; nrows is R except in an image's last group
-    const int ring = i0 + (nrows == R ? jc / R : jc / nrows);
+    const int rc = nrows == R ? jc / R : jc / nrows, ring = c.i0 + rc;
     const int i = nrows == R ? jc % R : jc % nrows;
-    const int4 rd = g.prings[ring];  // {N, offset in the sample buffer, natural-bin offset, log2(N/2)}
-    float2 *z = reinterpret_cast<float2 *>(smem + i * sample_stride(g.NSb) + rd.y);
+    const int bin0 = c.bin + rc * (H + 1);
+    float2 *z = reinterpret_cast<float2 *>(smem + i * sample_stride(g.NSb) + c.off + rc * c.stride);
     group_fft<H>(z, t, active, tws, g.M);
     if (active) {
       const int wstep = g.M / (2 * H);
@@ -110,8 +108,8 @@ __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a,
       for (int k = t; 2 * k <= H; k += T) {
         float2 xk, xhk;
         real_split_pair(z, H, k, tws[k * wstep], xk, xhk);
-        put_bin<OUT>(g, a, prow, s_kpos, ring, rd.z, row, k, xk);
-        if (2 * k != H) put_bin<OUT>(g, a, prow, s_kpos, ring, rd.z, row, H - k, xhk);
+        put_bin<OUT>(g, a, prow, s_kpos, ring, bin0, row, k, xk);
+        if (2 * k != H) put_bin<OUT>(g, a, prow, s_kpos, ring, bin0, row, H - k, xhk);
       }
     }
     __syncwarp();
@@ -129,8 +127,13 @@ __host__ __device__ inline int image_floats(const Geometry &g, int mode) {
   return (n + 3) & ~3;
 }
 
+// Threads of a CTA: with a bordered image and integer shifts one CTA of 16
+// warps fills an SM and takes as many rows as fit (launch_polar_t); otherwise
+// two of 8 warps.
+constexpr int polar_threads(int mode) { return mode == kPolarInt ? 512 : 256; }
+
 template <int R, int MODE, int OUT>
-__global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
+__global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
   extern __shared__ float4 smem_f4[];
   const int L = g.L, NS = g.NS, M = g.M;
   const int NSp = sample_stride(g.NSb);
@@ -147,7 +150,8 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
   const int NB16 = g.KS * 16;
   uint32_t *planes = reinterpret_cast<uint32_t *>(smem + R * NSp);
   if constexpr (OUT != kOutF32)
-    for (int idx = threadIdx.x; idx < R * NB16; idx += blockDim.x) planes[idx] = 0u;
+    for (int idx = threadIdx.x; idx < R * NB16 / 2; idx += blockDim.x)
+      reinterpret_cast<uint2 *>(planes)[idx] = make_uint2(0u, 0u);
   {
     const int *kp = OUT == kOutF32 ? g.kpos : g.kpos16;
     for (int k = threadIdx.x; k <= M / 2; k += blockDim.x) s_kpos[k] = kp[k];
@@ -220,16 +224,19 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
       // integer shifts: the bilinear weights of a sample do not depend on the
       // shift, which only moves the neighbourhood inside the bordered image
       const int Lp = g.pitch;
-      int soff[R];
-      bool run = nrows == R;  // the group's shifts step along x by one pixel
+      int soff[R];        // shift s = iy nx + ix is (smin + ix sstep, smin + iy sstep)
+      uint32_t step = 0;  // bit i: row i's shift is row i - 1's plus one pixel along x
+      {
+        int iy = s0 / g.nx, ix = s0 - iy * g.nx;
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        soff[i] = 0;
-        if (a.use_shifts && i < nrows) {
-          const float2 sh = g.shifts[s0 + i];
-          soff[i] = static_cast<int>(sh.y) * Lp + static_cast<int>(sh.x);
+        for (int i = 0; i < R; ++i) {
+          soff[i] = a.use_shifts ? (g.smin + iy * g.sstep) * Lp + g.smin + ix * g.sstep : 0;
+          if (i > 0 && ix > 0 && g.sstep == 1) step |= 1u << i;
+          if (++ix == g.nx) {
+            ix = 0;
+            ++iy;
+          }
         }
-        if (i > 0) run = run && soff[i] == soff[i - 1] + 1;
       }
       // eight samples per thread and pass, their tap loads issued together
       constexpr int QU = 8;
@@ -246,29 +253,23 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
           if (q < NS) {
             const int at = __float_as_int(tp[u].w);
             const float fx = tp[u].y, fy = tp[u].z, gx = 1.f - fx, gy = 1.f - fy;
-            const float *p = im + __float_as_int(tp[u].x) + soff[0];
+            const float *p = im + __float_as_int(tp[u].x);
             float *dst = smem + (at & 0xffff);
             auto put = [&](int i, float v) {
               dst[i * NSp] = v;
               if (OUT == kOutF32 && a.dbg_samples) a.dbg_samples[(row0 + i) * NS + (at >> 16)] = v;
             };
-            if (R > 1 && run) {  // neighbouring rows share the pixel columns between them
-              float t[R + 1], b[R + 1];
+            float t1 = 0.f, b1 = 0.f;  // the right-hand pixels of the row before
 #pragma unroll
-              for (int i = 0; i <= R; ++i) {
-                t[i] = p[i];
-                b[i] = p[Lp + i];
-              }
-#pragma unroll
-              for (int i = 0; i < R; ++i)
-                put(i, gy * (gx * t[i] + fx * t[i + 1]) + fy * (gx * b[i] + fx * b[i + 1]));
-            } else {
-#pragma unroll
-              for (int i = 0; i < R; ++i) {
-                if (i < nrows) {
-                  const float *pi = p + (soff[i] - soff[0]);
-                  put(i, gy * (gx * pi[0] + fx * pi[1]) + fy * (gx * pi[Lp] + fx * pi[Lp + 1]));
-                }
+            for (int i = 0; i < R; ++i) {
+              if (i < nrows) {
+                const float *pi = p + soff[i];
+                // a row whose shift is one pixel further along x starts at the columns the row before ended at
+                const bool next = (step >> i) & 1u;
+                const float t0 = next ? t1 : pi[0], b0 = next ? b1 : pi[Lp];
+                t1 = pi[1];
+                b1 = pi[Lp + 1];
+                put(i, gy * (gx * t0 + fx * t1) + fy * (gx * b0 + fx * b1));
               }
             }
           }
@@ -327,24 +328,11 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
     // warp, each transformed by a group of T threads (group_fft).
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     int fw = 0;  // warp that takes the first pass of the next class
-    for (int i1 = g.NR; i1 > 0;) {
-      const int H = g.rings[i1 - 1].x >> 1;
-      int i0 = i1 - 1;
-      while (i0 > 0 && (g.rings[i0 - 1].x >> 1) == H) --i0;
-#define MRA_RING_CLASS(HH) \
-    fw = ring_class<HH, R, OUT>(g, a, smem, planes, NB16, tws, s_kpos, i0, i1, nrows, row0, warp, lane, nwarps, fw)
-      switch (H) {
-        case 4: MRA_RING_CLASS(4); break;
-        case 8: MRA_RING_CLASS(8); break;
-        case 16: MRA_RING_CLASS(16); break;
-        case 32: MRA_RING_CLASS(32); break;
-        case 64: MRA_RING_CLASS(64); break;
-        case 128: MRA_RING_CLASS(128); break;
-        default: MRA_RING_CLASS(256); break;
-      }
-#undef MRA_RING_CLASS
-      i1 = i0;
-    }
+    sfor<0, kRingClasses>([&](auto kk) {  // longest first; a class the geometry lacks has no jobs
+      constexpr int k = decltype(kk)::value;
+      fw = ring_class<(256 >> k), R, OUT>(g, a, smem, planes, NB16, tws, s_kpos, g.cls[k], nrows, row0, warp, lane,
+                                          nwarps, fw);
+    });
 
     // Phase 3 (16-bit paths): copy-out in the layout of the tensor-core
     // kernel, 16 bytes per store.
@@ -374,33 +362,38 @@ __global__ void __launch_bounds__(256, 2) polar_fft_kernel(Geometry g, const __g
   }
 }
 
+inline cudaError_t polar_sms(int *sms) {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+  }
+  *sms = n;
+  return cudaSuccess;
+}
+
 template <int R, int MODE, int OUT>
 static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t smem, cudaStream_t st) {
   static size_t granted = 0;
   cudaError_t e = raise_smem_limit(polar_fft_kernel<R, MODE, OUT>, smem, granted);
   if (e != cudaSuccess) return e;
   // CTAs per image (each walks its share of the image's shift groups and
-  // stages the image once): four when two or more CTAs fit on an SM, so
-  // that the CTAs stay short and the last wave small; one when a CTA fills
-  // an SM, where the image staging would not overlap other work; more when
-  // the images are too few for about four waves of two CTAs per SM.
-  // (Measured on GB300: L = 76, 2 CTAs per SM: 1 / 2 / 4 per image 22.8 /
-  // 21.4 / 20.7 ms per 8192 images; L = 128, 1 CTA per SM: 1 / 2 per image
-  // 51.7 / 57.3 ms per 2048 images.)
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  // stages the image once): four of the small CTAs, so that the last wave
+  // stays small, one of those that fill an SM; more when the images are too
+  // few for four waves.
+  int sms = 0;
+  e = polar_sms(&sms);
+  if (e != cudaSuccess) return e;
+  constexpr int kPerSm = 512 / polar_threads(MODE);
   const int64_t groups = (a.rows_per_img + R - 1) / R;
-  const int64_t want = (static_cast<int64_t>(8) * sms + a.n_imgs - 1) / a.n_imgs;
-  int64_t per_img = smem + 1024 <= 232448 / 2 ? 4 : 1;
+  const int64_t want = (static_cast<int64_t>(4 * kPerSm) * sms + a.n_imgs - 1) / a.n_imgs;
+  int64_t per_img = kPerSm > 1 && smem + 1024 <= 232448 / 2 ? 4 : 1;
   if (per_img < want) per_img = want;
   if (per_img > groups) per_img = groups;
   dim3 grid(static_cast<unsigned>(per_img), static_cast<unsigned>(a.n_imgs));
-  polar_fft_kernel<R, MODE, OUT><<<grid, 256, smem, st>>>(g, a);
+  polar_fft_kernel<R, MODE, OUT><<<grid, polar_threads(MODE), smem, st>>>(g, a);
   return cudaGetLastError();
 }
 
@@ -415,26 +408,68 @@ inline size_t polar_smem_bytes(const Geometry &g, int mode, bool out16, int R) {
   return fixed + per_row * R;
 }
 
-// Rows (shifts) per CTA: as many as let two CTAs fit on an SM (~110 KB), else
-// as many as fit in 200 KB.
+// Most rows (shifts) per CTA: bordered integer grids as many as fit an SM, at
+// most 8; the others as many as let two CTAs fit (~110 KB), else as many as
+// fit in 200 KB, at most 4.
 inline int polar_cta_rows(const Geometry &g, int mode, bool out16) {
   const size_t fixed = polar_smem_bytes(g, mode, out16, 0);
   const size_t per_row = polar_smem_bytes(g, mode, out16, 1) - fixed;
-  int R = static_cast<int>((112640 > fixed ? 112640 - fixed : 0) / per_row);
-  if (R < 1) R = static_cast<int>((204800 > fixed ? 204800 - fixed : 0) / per_row);
-  return R < 1 ? 1 : (R > 4 ? 4 : R);
+  auto fit = [&](size_t bytes) { return static_cast<int>((bytes > fixed ? bytes - fixed : 0) / per_row); };
+  int R = mode == kPolarInt ? fit(kMaxSmemPerBlock) : fit(112640);
+  if (R < 1) R = fit(204800);
+  const int most = mode == kPolarInt ? 8 : 4;
+  return R < 1 ? 1 : (R > most ? most : R);
+}
+
+// Rows per CTA of a bordered integer grid.  A group of R rows takes about
+// R + 2.5 row times (its phases' latency and barriers; fitted to R = 2..8 on
+// the 76-, 90- and 128-pixel workloads: 12,000 images of 76 px, 81 shifts,
+// 16-bit output: R = 2 28.4 ms, 3 23.8, 4 20.0, 5 19.0, and 21.4 for two CTAs
+// of 8 warps with 2 rows each), so large groups win on long stacks, where they
+// also share table entries and pixel columns, and one row per CTA on calls
+// whose rows do not fill the SMs.
+inline int polar_int_rows(const PolarArgs &a, int most, int sms) {
+  int best = 1;
+  double best_cost = 1e300;
+  for (int R = 1; R <= most; ++R) {
+    if (R == 7) continue;  // not instantiated
+    const int64_t groups = a.n_imgs * ((a.rows_per_img + R - 1) / R);
+    const double cost = static_cast<double>((groups + sms - 1) / sms) * (R + 2.5);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = R;
+    }
+  }
+  return best;
 }
 
 template <int MODE, int OUT>
 static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
   int R = polar_cta_rows(g, MODE, OUT != kOutF32);
   if (R > a.rows_per_img) R = a.rows_per_img;
-  const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
-  switch (R) {
-    case 1: return launch_polar_r<1, MODE, OUT>(g, a, smem, st);
-    case 2: return launch_polar_r<2, MODE, OUT>(g, a, smem, st);
-    case 3: return launch_polar_r<3, MODE, OUT>(g, a, smem, st);
-    default: return launch_polar_r<4, MODE, OUT>(g, a, smem, st);
+  if constexpr (MODE == kPolarInt) {
+    int sms = 0;
+    const cudaError_t e = polar_sms(&sms);
+    if (e != cudaSuccess) return e;
+    R = polar_int_rows(a, R, sms);
+    const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
+    switch (R) {
+      case 1: return launch_polar_r<1, MODE, OUT>(g, a, smem, st);
+      case 2: return launch_polar_r<2, MODE, OUT>(g, a, smem, st);
+      case 3: return launch_polar_r<3, MODE, OUT>(g, a, smem, st);
+      case 4: return launch_polar_r<4, MODE, OUT>(g, a, smem, st);
+      case 5: return launch_polar_r<5, MODE, OUT>(g, a, smem, st);
+      case 6: return launch_polar_r<6, MODE, OUT>(g, a, smem, st);
+      default: return launch_polar_r<8, MODE, OUT>(g, a, smem, st);
+    }
+  } else {
+    if (R == 3) R = 2;
+    const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
+    switch (R) {
+      case 1: return launch_polar_r<1, MODE, OUT>(g, a, smem, st);
+      case 2: return launch_polar_r<2, MODE, OUT>(g, a, smem, st);
+      default: return launch_polar_r<4, MODE, OUT>(g, a, smem, st);
+    }
   }
 }
 
