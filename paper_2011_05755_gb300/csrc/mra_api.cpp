@@ -542,16 +542,13 @@ int build_tables(mra_handle *h) {
     g.NSb = NS;
     g.pad = g.pitch = 0;
     const int out16 = h->half;
-    const int bare_rows = mra::polar_rows_per_cta(g, mra::kPolarBare, out16);
     if (need <= 8) {
       mra::Geometry t = g;
       const int mode = integral ? mra::kPolarInt : mra::kPolarFrac;
       t.pad = need <= 4 ? 4 : 8;  // a multiple of 4 keeps the interior float4-aligned
       t.pitch = c.L + 2 * t.pad;
-      // a fractional grid takes the border only where it costs no row of the CTA
-      const bool fits = integral || (mra::polar_smem_one_row(t, mode, out16) <= mra::kMaxSmemPerBlock &&
-                                     mra::polar_rows_per_cta(t, mode, out16) == bare_rows);
-      if (fits) {
+      // (an integral grid was checked with the widest border; a fractional one falls back to the bare image)
+      if (integral || mra::polar_smem_one_row(t, mode, out16) <= mra::kMaxSmemPerBlock) {
         g = t;
         g.mode = mode;
         // rows a multiple of 16 floats long (or nearly) put vertical neighbours in the same banks

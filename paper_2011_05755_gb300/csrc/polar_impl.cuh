@@ -127,10 +127,17 @@ __host__ __device__ inline int image_floats(const Geometry &g, int mode) {
   return (n + 3) & ~3;
 }
 
-// Threads of a CTA: with a bordered image and integer shifts one CTA of 16
-// warps fills an SM and takes as many rows as fit (launch_polar_t); otherwise
-// two of 8 warps.
-constexpr int polar_threads(int mode) { return mode == kPolarInt ? 512 : 256; }
+// Threads of a CTA: with a bordered image one CTA of 16 warps fills an SM and
+// takes as many rows as fit (launch_polar_t); otherwise two of 8 warps.
+constexpr int polar_threads(int mode) { return mode != kPolarBare ? 512 : 256; }
+
+// Bilinear interpolation with the fused multiply-adds written out: left to
+// the compiler, instantiations with different row counts fuse differently,
+// and an image's last bits would depend on the size of its call.
+__device__ __forceinline__ float bilerp(float fx, float fy, float gx, float gy, float t0, float t1, float b0, float b1) {
+  const float t = fmaf(gx, t0, __fmul_rn(fx, t1)), b = fmaf(gx, b0, __fmul_rn(fx, b1));
+  return fmaf(gy, t, __fmul_rn(fy, b));
+}
 
 template <int R, int MODE, int OUT>
 __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
@@ -269,7 +276,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
                 const float t0 = next ? t1 : pi[0], b0 = next ? b1 : pi[Lp];
                 t1 = pi[1];
                 b1 = pi[Lp + 1];
-                put(i, gy * (gx * t0 + fx * t1) + fy * (gx * b0 + fx * b1));
+                put(i, bilerp(fx, fy, gx, gy, t0, t1, b0, b1));
               }
             }
           }
@@ -290,7 +297,6 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
       if constexpr (MODE == kPolarFrac) {
         const int Lp = g.pitch;
         const float *im0 = im + g.pad * Lp + g.pad;  // pixel (0, 0)
-#pragma unroll 4
         for (int q = threadIdx.x; q < NS; q += blockDim.x) {
           const float4 tp = __ldg(g.taps + q);  // {place, offset x, offset y}
           const int at = __float_as_int(tp.x);
@@ -301,7 +307,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
               const float xf = floorf(x), yf = floorf(y);
               const float fx = x - xf, fy = y - yf, gx = 1.f - fx, gy = 1.f - fy;
               const float *p = im0 + static_cast<int>(yf) * Lp + static_cast<int>(xf);
-              const float v = gy * (gx * p[0] + fx * p[1]) + fy * (gx * p[Lp] + fx * p[Lp + 1]);
+              const float v = bilerp(fx, fy, gx, gy, p[0], p[1], p[Lp], p[Lp + 1]);
               smem[i * NSp + (at & 0xffff)] = v;
               if (OUT == kOutF32 && a.dbg_samples) a.dbg_samples[(row0 + i) * NS + (at >> 16)] = v;
             }
@@ -408,27 +414,28 @@ inline size_t polar_smem_bytes(const Geometry &g, int mode, bool out16, int R) {
   return fixed + per_row * R;
 }
 
-// Most rows (shifts) per CTA: bordered integer grids as many as fit an SM, at
-// most 8; the others as many as let two CTAs fit (~110 KB), else as many as
+// Most rows (shifts) per CTA: with a bordered image as many as fit an SM, at
+// most 8; otherwise as many as let two CTAs fit (~110 KB), else as many as
 // fit in 200 KB, at most 4.
 inline int polar_cta_rows(const Geometry &g, int mode, bool out16) {
   const size_t fixed = polar_smem_bytes(g, mode, out16, 0);
   const size_t per_row = polar_smem_bytes(g, mode, out16, 1) - fixed;
   auto fit = [&](size_t bytes) { return static_cast<int>((bytes > fixed ? bytes - fixed : 0) / per_row); };
-  int R = mode == kPolarInt ? fit(kMaxSmemPerBlock) : fit(112640);
+  int R = mode != kPolarBare ? fit(kMaxSmemPerBlock) : fit(112640);
   if (R < 1) R = fit(204800);
-  const int most = mode == kPolarInt ? 8 : 4;
+  const int most = mode != kPolarBare ? 8 : 4;
   return R < 1 ? 1 : (R > most ? most : R);
 }
 
-// Rows per CTA of a bordered integer grid.  A group of R rows takes about
+// Rows per CTA with a bordered image.  A group of R rows takes about
 // R + 2.5 row times (its phases' latency and barriers; fitted to R = 2..8 on
 // the 76-, 90- and 128-pixel workloads: 12,000 images of 76 px, 81 shifts,
 // 16-bit output: R = 2 28.4 ms, 3 23.8, 4 20.0, 5 19.0, and 21.4 for two CTAs
-// of 8 warps with 2 rows each), so large groups win on long stacks, where they
+// of 8 warps with 2 rows each; 5,003 images of 32 px on a half-pixel grid of
+// 49: 4 rows 1.92 ms, 6 1.47, 8 1.35, two small CTAs with 4 rows each 1.77), so large groups win on long stacks, where they
 // also share table entries and pixel columns, and one row per CTA on calls
 // whose rows do not fill the SMs.
-inline int polar_int_rows(const PolarArgs &a, int most, int sms) {
+inline int polar_bordered_rows(const PolarArgs &a, int most, int sms) {
   int best = 1;
   double best_cost = 1e300;
   for (int R = 1; R <= most; ++R) {
@@ -447,11 +454,11 @@ template <int MODE, int OUT>
 static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStream_t st) {
   int R = polar_cta_rows(g, MODE, OUT != kOutF32);
   if (R > a.rows_per_img) R = a.rows_per_img;
-  if constexpr (MODE == kPolarInt) {
+  if constexpr (MODE != kPolarBare) {
     int sms = 0;
     const cudaError_t e = polar_sms(&sms);
     if (e != cudaSuccess) return e;
-    R = polar_int_rows(a, R, sms);
+    R = polar_bordered_rows(a, R, sms);
     const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
     switch (R) {
       case 1: return launch_polar_r<1, MODE, OUT>(g, a, smem, st);
