@@ -17,7 +17,8 @@ constexpr int kRescoreThreads = 256;  // 8 warps per CTA (one image)
 // FP32 rescore: for each candidate row of an image, resample at its shift,
 // ring-FFT, contract with its reference in FP32, inverse DFT; keep the best
 // (value, smallest index) over the candidates' angles as the argmax key.
-// One CTA per image.
+// One CTA per image, or several (gridDim.y) that take its candidates in turn
+// when the images alone would not fill the SMs.
 // ---------------------------------------------------------------------------
 // Registers are held to 64 per thread for M = 32..256, so that four CTAs
 // (images) fit on an SM where their shared memory allows (the 76-pixel
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(kRescoreThreads, (M >= 32 && M <= 256) ? 4 : 1
   // read by the inverse DFT, and warp 0 joins the barrier after resampling
   // only once its inverse DFT is done, before the spectrum buffer is
   // rewritten).
-  for (int c = 0; c < kTopRows; ++c) {
+  for (int c = blockIdx.y; c < kTopRows; c += gridDim.y) {
     const int rowid = a.cand[img * kTopRows + c];
     if (rowid < 0) continue;  // uniform over the CTA
     const int m = rowid & 1;
@@ -211,7 +212,12 @@ __global__ void __launch_bounds__(kRescoreThreads, (M >= 32 && M <= 256) ? 4 : 1
       if (lane == 0 && key > best) best = key;
     }
   }
-  if (threadIdx.x == 0) a.best[img] = best;
+  if (threadIdx.x == 0) {
+    if (gridDim.y == 1)
+      a.best[img] = best;
+    else if (best)
+      atomicMax(a.best + img, best);
+  }
 }
 
 size_t rescore_smem(const Geometry &g) {
@@ -234,7 +240,22 @@ static cudaError_t launch_rescore_t(const Geometry &g, const RescoreArgs &a, cud
   const size_t smem = rescore_smem(g);
   cudaError_t e = rescore_smem_attr<M>(smem);
   if (e != cudaSuccess) return e;
-  rescore_kernel<M><<<static_cast<unsigned>(a.n), kRescoreThreads, smem, st>>>(g, a);
+  // CTAs per image: as many (1, 2, 4, 8) as still run at once.  Each stages
+  // the image again, so only calls that leave SMs idle are split (top-8 and
+  // rescore together: one image of 64 px 131 -> 27 us, 200 images of 76 px 241
+  // -> 112 us).
+  static int at_once = 0;
+  if (at_once == 0) {
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    at_once = sms;
+  }
+  const int64_t slots = static_cast<int64_t>(at_once) * (2 * smem + 2048 > 233472 ? 1 : (4 * smem + 4096 > 233472 ? 2 : 4));
+  unsigned parts = 1;
+  while (parts < kTopRows && a.n * parts * 2 <= slots) parts *= 2;
+  rescore_kernel<M><<<dim3(static_cast<unsigned>(a.n), parts), kRescoreThreads, smem, st>>>(g, a);
   return cudaGetLastError();
 }
 

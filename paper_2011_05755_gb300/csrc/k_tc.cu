@@ -574,56 +574,110 @@ __global__ void __launch_bounds__(TcShape<M, KT>::THREADS) cc_tc_kernel(Geometry
 
 // ---------------------------------------------------------------------------
 // Top-8 rows (reference, shift, mirror) per image by row maximum; ties keep
-// the smaller row index.  One warp per image.
+// the smaller row index.  One CTA per image, three steps: the maximum of each
+// thread's values (float4 loads, all in flight), a threshold (the eighth
+// largest of the thread maxima: eight values reach it, so the eight largest
+// do), and the rows that reach it, collected and ordered by one warp.  Also
+// clears the image's argmax key.  Bound by the latency of the loads; against
+// one warp per image walking all rows with a sorted list, top-8 and rescore
+// together: 12,000 images of 16,200 rows 5.80 -> 5.05 ms, 6,000 of 49,000 rows
+// 3.62 -> 2.72 ms.
 // ---------------------------------------------------------------------------
-__global__ void top8_kernel(const float *__restrict__ rowmax, int64_t n, int nrows, int *cand) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t img = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
-  if (img >= n) return;
-  float v[kTopRows];
-  int id[kTopRows];
-#pragma unroll
+constexpr int kTopThreads = 256;
+constexpr int kTopList = 256;
+
+__global__ void __launch_bounds__(kTopThreads) top8_kernel(const float *__restrict__ rowmax, int nrows, int *cand,
+                                                           unsigned long long *best) {
+  __shared__ float s_top[kTopThreads / 32][kTopRows];
+  __shared__ unsigned long long s_list[kTopList];
+  __shared__ int s_count;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t img = blockIdx.x;
+  const float *rm = rowmax + img * nrows;  // nrows is even: 8-byte aligned
+  const float2 *rm2 = reinterpret_cast<const float2 *>(rm);
+  float m = -INFINITY;
+#pragma unroll 8
+  for (int j = tid; j < nrows / 2; j += kTopThreads) {
+    const float2 v = __ldg(rm2 + j);
+    m = fmaxf(m, fmaxf(v.x, v.y));
+  }
+  if (tid == 0) {
+    s_count = 0;
+    best[img] = 0ull;
+  }
+  // the eight largest of each warp's thread maxima, then of those
+  float t = m;
   for (int e = 0; e < kTopRows; ++e) {
-    v[e] = -INFINITY;
-    id[e] = 0x7fffffff;
-  }
-  const float *rm = rowmax + img * nrows;
-  for (int j = lane; j < nrows; j += 32) {
-    const float x = rm[j];
-    if (x > v[kTopRows - 1]) {
-      v[kTopRows - 1] = x;
-      id[kTopRows - 1] = j;
+    float x = t;
 #pragma unroll
-      for (int e = kTopRows - 1; e > 0; --e)
-        if (v[e] > v[e - 1]) {
-          const float tv = v[e];
-          v[e] = v[e - 1];
-          v[e - 1] = tv;
-          const int ti = id[e];
-          id[e] = id[e - 1];
-          id[e - 1] = ti;
+    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if (lane == 0) s_top[warp][e] = x;
+    if (lane == __ffs(__ballot_sync(0xffffffffu, t == x)) - 1) t = -INFINITY;
+  }
+  __syncthreads();
+  float thr = -INFINITY;
+  {
+    float u = s_top[lane >> 3][lane & 7], w = s_top[4 + (lane >> 3)][lane & 7];  // 64 values, two per lane
+    for (int e = 0; e < kTopRows; ++e) {
+      float x = fmaxf(u, w);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+      thr = x;
+      if (lane == __ffs(__ballot_sync(0xffffffffu, fmaxf(u, w) == x)) - 1) (u >= w ? u : w) = -INFINITY;
+    }
+  }
+  if (m > -INFINITY && m >= thr) {
+    for (int j = tid; j < nrows / 2; j += kTopThreads) {
+      const float2 v = __ldg(rm2 + j);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float x = e ? v.y : v.x;
+        if (x > -INFINITY && x >= thr) {
+          const int at = atomicAdd(&s_count, 1);
+          if (at < kTopList) s_list[at] = make_key(x, static_cast<uint32_t>(2 * j + e));
         }
+      }
     }
   }
-  for (int round = 0; round < kTopRows; ++round) {
-    unsigned long long key = (v[0] == -INFINITY) ? 0ull : make_key(v[0], static_cast<uint32_t>(id[0]));
-    unsigned long long best = key;
+  __syncthreads();
+  if (warp > 0) return;
+  if (s_count <= kTopList) {
+    unsigned long long key[kTopList / 32];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
-      best = o > best ? o : best;
-    }
-    if (lane == 0) cand[img * kTopRows + round] = best ? static_cast<int>(0xffffffffu - static_cast<uint32_t>(best)) : -1;
-    const unsigned win = __ballot_sync(0xffffffffu, best != 0 && key == best);
-    if (best != 0 && lane == __ffs(win) - 1) {
+    for (int i = 0; i < kTopList / 32; ++i) key[i] = lane + 32 * i < s_count ? s_list[lane + 32 * i] : 0ull;
+    for (int round = 0; round < kTopRows; ++round) {
+      unsigned long long x = 0ull;
 #pragma unroll
-      for (int e = 0; e < kTopRows - 1; ++e) {
-        v[e] = v[e + 1];
-        id[e] = id[e + 1];
+      for (int i = 0; i < kTopList / 32; ++i) x = key[i] > x ? key[i] : x;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = y > x ? y : x;
       }
-      v[kTopRows - 1] = -INFINITY;
-      id[kTopRows - 1] = 0x7fffffff;
+#pragma unroll
+      for (int i = 0; i < kTopList / 32; ++i)
+        if (key[i] == x) key[i] = 0ull;  // keys are distinct
+      if (lane == 0)
+        cand[img * kTopRows + round] = x ? static_cast<int>(0xffffffffu - static_cast<uint32_t>(x)) : -1;
     }
+    return;
+  }
+  // more than kTopList rows share the threshold (equal maxima): each round's largest key below the last one
+  unsigned long long last = ~0ull;
+  for (int round = 0; round < kTopRows; ++round) {
+    unsigned long long x = 0ull;
+    for (int j = lane; j < nrows; j += 32) {
+      const float v = rm[j];
+      const unsigned long long k = v > -INFINITY ? make_key(v, static_cast<uint32_t>(j)) : 0ull;
+      if (k < last && k > x) x = k;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+      x = y > x ? y : x;
+    }
+    if (lane == 0) cand[img * kTopRows + round] = x ? static_cast<int>(0xffffffffu - static_cast<uint32_t>(x)) : -1;
+    last = x ? x : 0ull;
   }
 }
 
@@ -682,9 +736,10 @@ cudaError_t launch_cc_tc(const Geometry &g, const TcArgs &a, bool fp16, cudaStre
 #undef MRA_TC_CASE
 }
 
-cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, cudaStream_t st) {
+cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, unsigned long long *best,
+                        cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  top8_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, st>>>(rowmax, n, nrows, cand);
+  top8_kernel<<<static_cast<unsigned>(n), kTopThreads, 0, st>>>(rowmax, nrows, cand, best);
   return cudaGetLastError();
 }
 

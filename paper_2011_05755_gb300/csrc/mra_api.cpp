@@ -963,7 +963,7 @@ int align_chunk_half(mra_handle *h, const float *imgs, int64_t cnt, mra_pose_t *
   prof_end(h, rec, 1, st);
   if (rc) return rc;
   rec = prof_begin(h, MRA_STAGE_RESCORE, st);
-  rc = check_launch(h, mra::launch_top8(h->rowmax, cnt, h->K * h->g.S * 2, h->cand, st), "top-8 kernel");
+  rc = check_launch(h, mra::launch_top8(h->rowmax, cnt, h->K * h->g.S * 2, h->cand, h->best, st), "top-8 kernel");
   if (!rc) {
     mra::RescoreArgs r{};
     r.imgs = imgs;

@@ -147,7 +147,7 @@ struct RescoreArgs {
   int64_t n;
   const int *cand;               // [n][kTopRows] row ids (k * S + s) * 2 + m, or -1
   const float2 *B;               // FP32 weighted reference spectra, tiled
-  unsigned long long *best;      // [n] argmax keys (written)
+  unsigned long long *best;      // [n] argmax keys (zero on entry)
 };
 
 cudaError_t launch_refs16(const Geometry &g, const float2 *B, int ktiles, uint4 *B16, bool fp16, cudaStream_t st);
@@ -156,7 +156,8 @@ cudaError_t launch_cc_hybrid256(const Geometry &g, const TcArgs &a, bool fp16, c
 // M = 512: the same.
 cudaError_t launch_cc_hybrid512(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st);
 cudaError_t launch_cc_tc(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st);
-cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, cudaStream_t st);
+cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, unsigned long long *best,
+                        cudaStream_t st);  // (clears best)
 cudaError_t launch_rescore(const Geometry &g, const RescoreArgs &a, cudaStream_t st);
 size_t rescore_smem(const Geometry &g);
 int rescore_ctas_per_sm(const Geometry &g);  // resident rescore CTAs per SM (0 if unknown)
