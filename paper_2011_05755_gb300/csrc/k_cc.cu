@@ -33,13 +33,16 @@ namespace mra {
 
 int cc_threads_per_pair(int M) { return M >= 256 ? 16 : M / 16; }
 
-template <int M, int KT>
+// A tile is kTile rows x KT references; a lane owns 2 rows x RL references of
+// one slice of a frequency's bins.  The number of slices (2, at M = 512 4)
+// fixes the order in which a pair's bins are added.
+template <int M, int KT, int RL>
 struct CCShape {
   static constexpr int RT = kTile;                         // rows per tile
   static constexpr int PAIRS = RT * KT;
-  static constexpr int WARPS = (M >= 512) ? 8 : 16;        // 16 warps unless staging would not fit
+  static constexpr int WARPS = (M >= 512 || PAIRS < 64) ? 8 : 16;  // M = 512: 16 would not fit; 32 pairs: two CTAs per SM
   static constexpr int THREADS = 32 * WARPS;
-  static constexpr int LANES_PER_SLICE = (RT / 2) * (KT / 2);  // lane = 2 rows x 2 refs
+  static constexpr int LANES_PER_SLICE = (RT / 2) * (KT / RL);
   static constexpr int NSPLIT = 32 / LANES_PER_SLICE;          // bin slices per frequency
   static constexpr int P = IfftShape<M>::P;                    // float2 per pair buffer
   static constexpr size_t STATE = static_cast<size_t>(PAIRS) * P * sizeof(float2);
@@ -52,15 +55,15 @@ struct CCShape {
 
 // Bank swizzle of the per-pair spectrum buffers (an XOR below T, so the
 // inverse DFT's reads stay one base plus constant offsets).
-template <int M, int KT>
+template <int M, int KT, int RL>
 __device__ __forceinline__ int pair_swz(int p) {
   const int row = p / KT, ref = p % KT;
-  return (row * (KT / 2) + (ref >> 1)) & (IfftShape<M>::T - 1);
+  return (RL == 2 ? row * (KT / 2) + (ref >> 1) : (row >> 1) * KT + ref) & (IfftShape<M>::T - 1);
 }
 
-template <int M, int KT>
-__global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geometry g, CCArgs a) {
-  using Sh = CCShape<M, KT>;
+template <int M, int KT, int RL>
+__global__ void __launch_bounds__(CCShape<M, KT, RL>::THREADS) cc_fp32_kernel(Geometry g, CCArgs a) {
+  using Sh = CCShape<M, KT, RL>;
   constexpr int T = IfftShape<M>::T;
   constexpr int U = IfftShape<M>::U;
   extern __shared__ float4 smem_f4[];
@@ -90,11 +93,11 @@ __global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geomet
     const int slice = lane / Sh::LANES_PER_SLICE;
     const int li = lane % Sh::LANES_PER_SLICE;
     const int rp = li % (Sh::RT / 2);   // rows 2rp, 2rp+1
-    const int kp = li / (Sh::RT / 2);   // refs 2kp, 2kp+1 of the tile
+    const int kp = li / (Sh::RT / 2);   // refs RL kp .. RL kp + RL - 1 of the tile
     const int ref0 = kt * KT;
     const float2 *Atile = a.A + rt * g.NB * kTile;
     const float2 *Btile = a.B + static_cast<int64_t>(ref0 / kTile) * g.NB * kTile;
-    const int bsub = (ref0 % kTile) / 2 + kp;  // float4 index of this lane's 2 refs within a bin
+    const int bsub = (ref0 % kTile) / RL + kp;  // index of this lane's refs (RL float2) within a bin
     float4 *stA = reinterpret_cast<float4 *>(stage0 + warp * stage_bytes);
     float4 *stB = reinterpret_cast<float4 *>(stage0 + warp * stage_bytes + stage_bytes / 2);
     uint64_t *bar = bars + warp;
@@ -119,28 +122,35 @@ __global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geomet
         break;
       }
       phase ^= 1u;
-      float p1[4] = {0.f, 0.f, 0.f, 0.f}, p2[4] = {0.f, 0.f, 0.f, 0.f};
-      float p3[4] = {0.f, 0.f, 0.f, 0.f}, p4[4] = {0.f, 0.f, 0.f, 0.f};
+      constexpr int kAcc = 2 * RL;
+      float p1[kAcc] = {}, p2[kAcc] = {}, p3[kAcc] = {}, p4[kAcc] = {};
 #pragma unroll 4
       for (int b = slice; b < seg.y; b += Sh::NSPLIT) {
         const float4 av = stA[b * (kTile / 2) + rp];
-        const float4 bv = stB[b * (kTile / 2) + bsub];
+        float2 bv[RL];
+        if constexpr (RL == 2) {
+          const float4 b4 = stB[b * (kTile / 2) + bsub];
+          bv[0] = make_float2(b4.x, b4.y);
+          bv[1] = make_float2(b4.z, b4.w);
+        } else {
+          bv[0] = reinterpret_cast<const float2 *>(stB)[b * kTile + bsub];
+        }
         const float ar[2] = {av.x, av.z}, ai[2] = {av.y, av.w};
-        const float br[2] = {bv.x, bv.z}, bi[2] = {bv.y, bv.w};
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            p1[2 * i + j] = fmaf(ar[i], br[j], p1[2 * i + j]);
-            p2[2 * i + j] = fmaf(ai[i], bi[j], p2[2 * i + j]);
-            p3[2 * i + j] = fmaf(ar[i], bi[j], p3[2 * i + j]);
-            p4[2 * i + j] = fmaf(ai[i], br[j], p4[2 * i + j]);
+          for (int j = 0; j < RL; ++j) {
+            const int q = RL * i + j;
+            p1[q] = fmaf(ar[i], bv[j].x, p1[q]);
+            p2[q] = fmaf(ai[i], bv[j].y, p2[q]);
+            p3[q] = fmaf(ar[i], bv[j].y, p3[q]);
+            p4[q] = fmaf(ai[i], bv[j].x, p4[q]);
           }
       }
 #pragma unroll
       for (int off = 16; off >= Sh::LANES_PER_SLICE; off >>= 1)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kAcc; ++q) {
           p1[q] += __shfl_xor_sync(0xffffffffu, p1[q], off);
           p2[q] += __shfl_xor_sync(0xffffffffu, p2[q], off);
           p3[q] += __shfl_xor_sync(0xffffffffu, p3[q], off);
@@ -150,10 +160,10 @@ __global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geomet
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int p = (2 * rp + i) * KT + 2 * kp + j;
-            const int sw = pair_swz<M, KT>(p);
-            const int q = 2 * i + j;
+          for (int j = 0; j < RL; ++j) {
+            const int p = (2 * rp + i) * KT + RL * kp + j;
+            const int sw = pair_swz<M, KT, RL>(p);
+            const int q = RL * i + j;
             float2 *zp = Zs + p * Sh::P;
             // Z(f) = C_u + i C'
             zp[f ^ sw] = make_float2((p1[q] + p2[q]) - (p3[q] + p4[q]), (p3[q] - p4[q]) + (p1[q] - p2[q]));
@@ -179,7 +189,7 @@ __global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geomet
     const int ref = kt * KT + pc % KT;
     const bool valid = in_tile && row < a.rows && ref < a.K;
     float2 *zp = Zs + pc * Sh::P;
-    const int sw = pair_swz<M, KT>(pc);
+    const int sw = pair_swz<M, KT, RL>(pc);
 
     float2 y[IfftShape<M>::KK][T];
     pair_ifft<M>(zp, sw, zp, t, in_tile, tw, y);
@@ -232,41 +242,47 @@ __global__ void __launch_bounds__(CCShape<M, KT>::THREADS) cc_fp32_kernel(Geomet
   }
 }
 
-template <int M, int KT>
+template <int M, int KT, int RL>
 static cudaError_t launch_cc_t(const Geometry &g, const CCArgs &a, cudaStream_t st) {
-  using Sh = CCShape<M, KT>;
+  using Sh = CCShape<M, KT, RL>;
   const size_t smem = Sh::smem(a.seg_max);
   static size_t granted = 0;
-  cudaError_t e = raise_smem_limit(cc_fp32_kernel<M, KT>, smem, granted);
+  cudaError_t e = raise_smem_limit(cc_fp32_kernel<M, KT, RL>, smem, granted);
   if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + Sh::RT - 1) / Sh::RT;
   const int ref_tiles = (a.K + KT - 1) / KT;
   if (row_tiles <= 0) return cudaSuccess;
   dim3 grid(ref_tiles, static_cast<unsigned>(row_tiles));
-  cc_fp32_kernel<M, KT><<<grid, Sh::THREADS, smem, st>>>(g, a);
+  cc_fp32_kernel<M, KT, RL><<<grid, Sh::THREADS, smem, st>>>(g, a);
   return cudaGetLastError();
 }
 
 size_t cc_fp32_smem(int M, int seg_max) {
   switch (M) {
-    case 16: return CCShape<16, 8>::smem(seg_max);
-    case 32: return CCShape<32, 8>::smem(seg_max);
-    case 64: return CCShape<64, 8>::smem(seg_max);
-    case 128: return CCShape<128, 8>::smem(seg_max);
-    case 256: return CCShape<256, 8>::smem(seg_max);
-    case 512: return CCShape<512, 4>::smem(seg_max);
+    case 16: return CCShape<16, 8, 2>::smem(seg_max);
+    case 32: return CCShape<32, 8, 2>::smem(seg_max);
+    case 64: return CCShape<64, 8, 2>::smem(seg_max);
+    case 128: return CCShape<128, 8, 2>::smem(seg_max);
+    case 256: return CCShape<256, 8, 2>::smem(seg_max);
+    case 512: return CCShape<512, 4, 2>::smem(seg_max);
     default: return 0;
   }
 }
 
 cudaError_t launch_cc_fp32(const Geometry &g, const CCArgs &a, cudaStream_t st) {
   switch (g.M) {
-    case 16: return launch_cc_t<16, 8>(g, a, st);
-    case 32: return launch_cc_t<32, 8>(g, a, st);
-    case 64: return launch_cc_t<64, 8>(g, a, st);
-    case 128: return launch_cc_t<128, 8>(g, a, st);
-    case 256: return launch_cc_t<256, 8>(g, a, st);
-    case 512: return launch_cc_t<512, 4>(g, a, st);
+    case 16: return launch_cc_t<16, 8, 2>(g, a, st);
+    case 32: return launch_cc_t<32, 8, 2>(g, a, st);
+    case 64: return launch_cc_t<64, 8, 2>(g, a, st);
+    case 128: return launch_cc_t<128, 8, 2>(g, a, st);
+    case 256:
+      // 8 x 8 tiles, one CTA of 16 warps per SM, or 8 x 4 tiles, two of 8 warps:
+      // 15.5 against 18.4 ms at K = 100 (13 and 25 tiles per row tile), 349
+      // against 331 us at K = 10 (2 and 3), 1.98 against 1.33 ms at K = 1 (1 and
+      // 1): a small tile costs 0.62 of a large one, so it is taken where it
+      // leaves out enough padding references (K <= 4, 9..12)
+      return 0.62 * ((a.K + 3) / 4) < (a.K + 7) / 8 ? launch_cc_t<256, 4, 1>(g, a, st) : launch_cc_t<256, 8, 2>(g, a, st);
+    case 512: return launch_cc_t<512, 4, 2>(g, a, st);
     default: return cudaErrorInvalidValue;
   }
 }
