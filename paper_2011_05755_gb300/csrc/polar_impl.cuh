@@ -80,17 +80,17 @@ __device__ __forceinline__ void put_bin(const Geometry &g, const PolarArgs &a, u
 // the layout the path needs (FP32 tiled, 16-bit q/p words, debug).  s_kpos
 // holds the per-frequency base of the output layout: bin (ring, k) goes to
 // s_kpos[k] + ring.
-template <int H, int R, int OUT>
+template <int H, int R, int OUT, int NWARPS>
 __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a, float *smem, uint32_t *planes,
                                           int NB16, const float2 *tws, const int *s_kpos, const RingClass &c, int nrows,
-                                          int64_t row0, int warp, int lane, int nwarps, int first_warp) {
+                                          int64_t row0, int warp, int lane, int first_warp) {
   constexpr int T = GroupFft<H>::T;
   constexpr int JPW = 32 / T;  // jobs per warp pass
   const int njobs = (c.i1 - c.i0) * nrows;
   const int t = lane % T;
   // warp passes of this class start after the previous class's last pass
-  const int wslot = (warp - first_warp + nwarps) % nwarps;
-  for (int j0 = wslot * JPW; j0 < njobs; j0 += nwarps * JPW) {
+  const int wslot = (warp - first_warp) & (NWARPS - 1);
+  for (int j0 = wslot * JPW; j0 < njobs; j0 += NWARPS * JPW) {
     const int job = j0 + lane / T;
     const bool active = job < njobs;
     const int jc = active ? job : j0;
@@ -114,7 +114,7 @@ __device__ __forceinline__ int ring_class(const Geometry &g, const PolarArgs &a,
     }
     __syncwarp();
   }
-  return (first_warp + (njobs + JPW - 1) / JPW) % nwarps;  // first warp of the next class
+  return (first_warp + (njobs + JPW - 1) / JPW) & (NWARPS - 1);  // first warp of the next class
 }
 
 // Shared-memory image: the bare image, sampled with bounds checks
@@ -129,7 +129,7 @@ __host__ __device__ inline int image_floats(const Geometry &g, int mode) {
 
 // Threads of a CTA: with a bordered image one CTA of 16 warps fills an SM and
 // takes as many rows as fit (launch_polar_t); otherwise two of 8 warps.
-constexpr int polar_threads(int mode) { return mode != kPolarBare ? 512 : 256; }
+__host__ __device__ constexpr int polar_threads(int mode) { return mode != kPolarBare ? 512 : 256; }
 
 // Bilinear interpolation with the fused multiply-adds written out: left to
 // the compiler, instantiations with different row counts fuse differently,
@@ -142,6 +142,7 @@ __device__ __forceinline__ float bilerp(float fx, float fy, float gx, float gy, 
 template <int R, int MODE, int OUT>
 __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
   extern __shared__ float4 smem_f4[];
+  constexpr int NT = polar_threads(MODE);
   const int L = g.L, NS = g.NS, M = g.M;
   const int NSp = sample_stride(g.NSb);
   const int LL = L * L;
@@ -157,11 +158,11 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   const int NB16 = g.KS * 16;
   uint32_t *planes = reinterpret_cast<uint32_t *>(smem + R * NSp);
   if constexpr (OUT != kOutF32)
-    for (int idx = threadIdx.x; idx < R * NB16 / 2; idx += blockDim.x)
+    for (int idx = threadIdx.x; idx < R * NB16 / 2; idx += NT)
       reinterpret_cast<uint2 *>(planes)[idx] = make_uint2(0u, 0u);
   {
     const int *kp = OUT == kOutF32 ? g.kpos : g.kpos16;
-    for (int k = threadIdx.x; k <= M / 2; k += blockDim.x) s_kpos[k] = kp[k];
+    for (int k = threadIdx.x; k <= M / 2; k += NT) s_kpos[k] = kp[k];
   }
   const float *src = a.imgs + img * LL;
   const bool vec = (L & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
@@ -180,18 +181,18 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   } else if constexpr (MODE != kPolarBare) {
     // zero the bordered buffer, then copy the interior (pad is a multiple of 4)
     const int Lp = g.pitch;
-    for (int i = threadIdx.x; i < image_floats(g, MODE) / 4; i += blockDim.x)
+    for (int i = threadIdx.x; i < image_floats(g, MODE) / 4; i += NT)
       reinterpret_cast<float4 *>(im)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     float *dst = im + g.pad * Lp + g.pad;
     if (vec) {
       const int W = L / 4;
-      for (int i = threadIdx.x; i < L * W; i += blockDim.x) {
+      for (int i = threadIdx.x; i < L * W; i += NT) {
         const int y = i / W, x4 = i - y * W;
         reinterpret_cast<float4 *>(dst + y * Lp)[x4] = __ldg(reinterpret_cast<const float4 *>(src + y * L) + x4);
       }
     } else {
-      for (int i = threadIdx.x; i < LL; i += blockDim.x) {
+      for (int i = threadIdx.x; i < LL; i += NT) {
         const int y = i / L, x = i - y * L;
         dst[y * Lp + x] = __ldg(src + i);
       }
@@ -199,12 +200,12 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   } else {
     if (vec) {
       const float4 *s4 = reinterpret_cast<const float4 *>(src);
-      for (int i = threadIdx.x; i < LL / 4; i += blockDim.x) reinterpret_cast<float4 *>(im)[i] = __ldg(s4 + i);
+      for (int i = threadIdx.x; i < LL / 4; i += NT) reinterpret_cast<float4 *>(im)[i] = __ldg(s4 + i);
     } else {
-      for (int i = threadIdx.x; i < LL; i += blockDim.x) im[i] = __ldg(src + i);
+      for (int i = threadIdx.x; i < LL; i += NT) im[i] = __ldg(src + i);
     }
   }
-  for (int i = threadIdx.x; i < M; i += blockDim.x) tws[i] = g.fwd_tw[i];
+  for (int i = threadIdx.x; i < M; i += NT) tws[i] = g.fwd_tw[i];
   if (tma) {
     __syncthreads();  // the barrier's initialisation is visible to every thread
     const bool ok = mbar_wait_bounded(ibar, 0, a.wait_limit);
@@ -247,16 +248,16 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
       }
       // eight samples per thread and pass, their tap loads issued together
       constexpr int QU = 8;
-      for (int q0 = threadIdx.x; q0 < NS; q0 += QU * blockDim.x) {
+      for (int q0 = threadIdx.x; q0 < NS; q0 += QU * NT) {
         float4 tp[QU];
 #pragma unroll
         for (int u = 0; u < QU; ++u) {
-          const int q = q0 + u * blockDim.x;
+          const int q = q0 + u * NT;
           tp[u] = q < NS ? __ldg(g.taps + q) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int u = 0; u < QU; ++u) {
-          const int q = q0 + u * blockDim.x;
+          const int q = q0 + u * NT;
           if (q < NS) {
             const int at = __float_as_int(tp[u].w);
             const float fx = tp[u].y, fy = tp[u].z, gx = 1.f - fx, gy = 1.f - fy;
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
       if constexpr (MODE == kPolarFrac) {
         const int Lp = g.pitch;
         const float *im0 = im + g.pad * Lp + g.pad;  // pixel (0, 0)
-        for (int q = threadIdx.x; q < NS; q += blockDim.x) {
+        for (int q = threadIdx.x; q < NS; q += NT) {
           const float4 tp = __ldg(g.taps + q);  // {place, offset x, offset y}
           const int at = __float_as_int(tp.x);
 #pragma unroll
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
           }
         }
       } else {
-        for (int q = threadIdx.x; q < NS; q += blockDim.x) {
+        for (int q = threadIdx.x; q < NS; q += NT) {
           const float2 o = g.offs[q];  // the bare mode's buffer is in ring order
 #pragma unroll
           for (int i = 0; i < R; ++i) {
@@ -332,12 +333,12 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
     // Phase 2: ring FFTs.  Rings of equal length form a contiguous class; the
     // (ring, row) jobs of a class are spread over the warps, 32 / T jobs per
     // warp, each transformed by a group of T threads (group_fft).
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int fw = 0;  // warp that takes the first pass of the next class
     sfor<0, kRingClasses>([&](auto kk) {  // longest first; a class the geometry lacks has no jobs
       constexpr int k = decltype(kk)::value;
-      fw = ring_class<(256 >> k), R, OUT>(g, a, smem, planes, NB16, tws, s_kpos, g.cls[k], nrows, row0, warp, lane,
-                                          nwarps, fw);
+      fw = ring_class<(256 >> k), R, OUT, polar_threads(MODE) / 32>(g, a, smem, planes, NB16, tws, s_kpos, g.cls[k],
+                                                                    nrows, row0, warp, lane, fw);
     });
 
     // Phase 3 (16-bit paths): copy-out in the layout of the tensor-core
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
     if constexpr (OUT != kOutF32) {
       __syncthreads();
       const int per_k = nrows * 4;
-      for (int idx = threadIdx.x; idx < g.KS * per_k; idx += blockDim.x) {
+      for (int idx = threadIdx.x; idx < g.KS * per_k; idx += NT) {
         const int kk = nrows == R ? idx / (4 * R) : idx / per_k;
         const int rem = idx - kk * per_k;
         const int i = rem >> 2, t = rem & 3;
