@@ -27,10 +27,11 @@
 // operands are BF16 (one rounding of 2 Re C, 2 Im C and of the matrices), the
 // sums FP32; no intermediate is rounded in between, and the whole angular
 // state never exists outside TMEM.  The zero frequency is added after the
-// maximum (a constant over the angles, FP32).  Angles 64 and 192 use the two
-// columns that are empty at j = 0 (sin 0): column 0 of Oo holds
-// -sum 2 Im C sin(pi f / 2) and column 0 of Oe gets Ee(64) from a third even
-// product (matrix X, one nonzero column).
+// maximum (a constant over the angles, FP32).  Angles 64 and 192 need Ee and Oo
+// at j = 64: column 0 of Oo, empty at j = 0 (sin 0), holds -sum 2 Im C sin(pi f
+// / 2), and Ee(64) is an alternating sum of the even 2 Re C that the contraction
+// warps form in FP32, each over its own frequencies, and the f = 0 warp adds up
+// (a fifth product for it took a fifth of the MMAs).
 //
 // What bounds it, and why this split.  Each (row, reference) pair needs all
 // 129 frequencies on chip at once, so a tile cannot exceed the pairs whose
@@ -41,19 +42,19 @@
 // the warps that use them (rings up to 36) or in shared memory, and the
 // reference fragments stream from L2 into a register ring ahead of their use.
 // Measured (GB300, 12,000 images of the 76-pixel, 100-reference, 81-shift
-// workload, contraction stage): 20.7 ms, against 66.9 ms for cc_tc256_kernel
+// workload, contraction stage): 20.0 ms, against 66.9 ms for cc_tc256_kernel
 // (all mma.sync, angular state in shared memory, whole chunks of both
 // operands staged behind CTA barriers) and about 77 ms for a tcgen05 kernel
 // that ran the contraction on tcgen05 as well (four frequencies block-diagonal
 // per MMA, two 16-point inverse-DFT stages with a TMEM drain each).  Bound:
-// shared-memory / L1 bandwidth and tensor issue together.  Without the
-// reference loads 19.7 ms, without 16 of the 20 tcgen05.mma 17.0, without
-// both 13.4; what is left is the contraction warps' own instruction stream.
-// Steps measured on the way: rows in shared memory instead of registers
-// 29.4 ms; one operand stage per parity instead of per tile 23.6; references
-// through a per-warp TMA buffer in shared memory 27.4; L1::no_allocate on the
-// reference loads 22.2; ring of 4 / 5 / 6 / 7 / 8 k-steps 22.9 / 23.9 / 20.7 /
-// 20.7 / 22.6.
+// shared-memory / L1 bandwidth, tensor issue and the contraction warps'
+// latency together.  With Ee(64) as a fifth product it took 20.7 ms, of which
+// the reference loads hid all but 1.0, 16 of the 20 MMAs all but 3.7, and both
+// together all but 7.3.  Steps measured on the way: rows in shared memory
+// instead of registers 29.4 ms; one operand stage per parity instead of per
+// tile 23.6; references through a per-warp TMA buffer in shared memory 27.4;
+// L1::no_allocate on the reference loads 22.2; ring of 4 / 5 / 6 / 7 k-steps
+// 20.7 / 20.3 / 20.0 / 20.1.
 //
 // Roles (16 warps, one persistent CTA per SM):
 //   warps 0-7    contract: warp w holds, for each parity, 8 frequencies
@@ -65,7 +66,7 @@
 //   warps 8-11   read the accumulators of their TMEM lane quarter and write
 //                the row maxima;
 //   warp 12      issues every tcgen05.mma (one lane);
-//   warp 13      contracts f = 0;
+//   warp 13      contracts f = 0 and adds up Ee(64);
 //   warp 14      copies the row fragments to shared memory (when they are
 //                there).
 // All waits are bounded; a wait that gives up raises a CTA abort flag and
@@ -87,9 +88,10 @@ constexpr int kContract = 8;                     // contraction warps
 constexpr uint32_t kOperand = 128 * 64 * 2;      // one operand of a parity: 128 rows x 64 frequencies
 constexpr uint32_t kZStage = 2 * kOperand;       // real and imaginary parts
 constexpr uint32_t kW = 64 * 64 * 2;             // one DFT matrix
-constexpr uint32_t kWBytes = kHyb256Mats * kW;   // Ee, Oe, X, Eo, Oo
+constexpr uint32_t kWBytes = kHyb256Mats * kW;   // Ee, Oe, Eo, Oo
 constexpr int kNumBars = 16;  // zfull[2] zempty[2] dfull[2] dempty[2] x0full[2] afull[2] aempty[2] fin, spare
-constexpr uint32_t kMisc = kWBytes + 2 * 64 * 4 + kNumBars * 8 + 16;
+// matrices, f = 0 terms, Ee(64) and its parts (two tiles each), barriers
+constexpr uint32_t kMisc = kWBytes + 2 * (64 + 128 + kContract * 128) * 4 + kNumBars * 8 + 16;
 // Operand stages: both parities of a tile together, two of them, when the row
 // fragments are in registers (one synchronisation per tile); beside row
 // fragments in shared memory there is room for one parity.
@@ -113,9 +115,11 @@ struct HybPattern {
 
 // One parity of one tile by one contraction warp.  fa(i) and fb(i) are the
 // row and reference fragments of k-step i, done(i) is called after their use.
-// out[part * 2 + correlation][block][word].
-template <class P, bool FP16, class FA, class FB, class Done>
-__device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, uint32_t (&out)[4][2][4]) {
+// out[part * 2 + correlation][block][word]; with SUM, ee[block][correlation] is
+// the sum of 2 Re C over the slots, the last slot's times `last`.
+template <class P, bool FP16, bool SUM, class FA, class FB, class Done>
+__device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, uint32_t (&out)[4][2][4],
+                                                float (&ee)[2][2], float last) {
   float keep[2][4];
   sfor<0, 8>([&](auto ss) {
     constexpr int s = decltype(ss)::value;
@@ -131,6 +135,11 @@ __device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, u
     for (int k = 0; k < 2; ++k) {
       float v[4];
       pair_sums(d[k], v);
+      if constexpr (SUM) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          ee[k][e] = s == 0 ? v[e] : (s < 7 ? ee[k][e] + v[e] : fmaf(v[e], last, ee[k][e]));
+      }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if constexpr (s & 1)
@@ -143,14 +152,14 @@ __device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, u
 }
 
 // Every angle of the 32 rows of a warp's TMEM lane quarter into the debug table (dst null: no store).
-__device__ __noinline__ void hybrid_debug_row(uint32_t d, int corr, float x0, float *dst) {
+__device__ __noinline__ void hybrid_debug_row(uint32_t d, int corr, float x0, float e64, float *dst) {
 #pragma unroll 1
   for (int n = 0; n < 64; ++n) {
     uint32_t r[4];
     for (int i = 0; i < 4; ++i) tmem_ld1(d + i * 64 + n, r[i]);
     tmem_ld_wait();
     const float E = __uint_as_float(r[0]), F = __uint_as_float(r[1]);
-    const float G = __uint_as_float(r[2]), H = __uint_as_float(r[3]);
+    const float G = n ? __uint_as_float(r[2]) : e64, H = __uint_as_float(r[3]);
     const float c[4] = {n ? (E + F) + (G + H) : E + F, n ? (E + F) - (G + H) : G + H,
                         n ? (E - F) + (G - H) : E - F, n ? (E - F) - (G - H) : G - H};
     const int at[4] = {n, n ? 256 - n : 64, 128 + n, n ? 128 - n : 192};
@@ -167,7 +176,7 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
   constexpr int T = P::kSteps;
   constexpr bool kRegs = PATTERN == 0;                     // row fragments in registers (104 per thread)
   constexpr int kZp = z_parities(PATTERN), kZs = z_stages(PATTERN);
-  constexpr int PF = kRegs ? 7 : 9;                        // k-steps of references in the register ring
+  constexpr int PF = kRegs ? 6 : 9;                        // k-steps of references in the register ring
   constexpr uint32_t kTile16 = P::KS * 512u;               // fragment bytes of a row or reference tile
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -175,7 +184,9 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
   unsigned char *sW = sZ + kZs * kZp * kZStage;            // DFT matrices
   unsigned char *sF = sW + kWBytes;                        // row fragments [KS][512] (pattern 1)
   float *s_x0 = reinterpret_cast<float *>(sF + (kRegs ? 0u : kTile16));  // [2][64] zero-frequency terms
-  uint64_t *bars = reinterpret_cast<uint64_t *>(s_x0 + 128);
+  float *s_e = s_x0 + 2 * 64;                              // [2][128] Ee(64)
+  float *s_part = s_e + 2 * 128;                           // [2][8 warps][128] its parts
+  uint64_t *bars = reinterpret_cast<uint64_t *>(s_part + 2 * kContract * 128);
   uint64_t *zfull = bars, *zempty = bars + 2, *dfull = bars + 4, *dempty = bars + 6, *x0full = bars + 8,
            *afull = bars + 10, *aempty = bars + 12, *fin = bars + 14;
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + kNumBars);
@@ -187,7 +198,7 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(zfull + s, kContract);
-      mbar_init(zempty + s, 1);
+      mbar_init(zempty + s, 2);  // the MMAs have read the operands, warp 13 the parts of Ee(64)
       mbar_init(dfull + s, 1);
       mbar_init(dempty + s, 4);
       mbar_init(x0full + s, 1);
@@ -241,23 +252,26 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
         auto parity = [&](auto pp) {
           constexpr int p = decltype(pp)::value;
           uint32_t out[4][2][4];
+          float ee[2][2];
+          // even f = 2 (8 s + warp) + 2; the last, f = 128, is its own mirror image
+          const float lastw = warp == 7 ? 0.5f : 1.f;
           // register ring: entry i % PF holds k-step i; refilled on use with
           // k-step i + PF, or with the first ones of the next parity
           const unsigned char *cur = bw + p * T * 512, *next = p ? bn : cur + T * 512;
           auto fb = [&](int i) { return b[i % PF]; };
           auto refill = [&](int i) { b[i % PF] = load_frag(i + PF < T ? cur + (i + PF) * 512 : next + i % PF * 512); };
           if constexpr (kRegs) {
-            contract_parity<P, FP16>([&](int i) { return ra[p * T + i]; }, fb,
-                                     [&](int i) {
-                                       refill(i);
-                                       if (last) ra[p * T + i] = load_frag(an + (p * T + i) * 512);
-                                     },
-                                     out);
+            contract_parity<P, FP16, p == 0>([&](int i) { return ra[p * T + i]; }, fb,
+                                             [&](int i) {
+                                               refill(i);
+                                               if (last) ra[p * T + i] = load_frag(an + (p * T + i) * 512);
+                                             },
+                                             out, ee, lastw);
           } else {
-            if (kt == k0 && !wait_or_abort(afull + p, un & 1, limit, abort, a.err)) return false;
+            if (kt == k0 && !warp_wait_or_abort(afull + p, un & 1, limit, abort, a.err)) return false;
             const unsigned char *sa = sF + woff + p * T * 512;
-            contract_parity<P, FP16>([&](int i) { return *reinterpret_cast<const uint4 *>(sa + i * 512); }, fb, refill,
-                                     out);
+            contract_parity<P, FP16, p == 0>([&](int i) { return *reinterpret_cast<const uint4 *>(sa + i * 512); }, fb,
+                                             refill, out, ee, lastw);
             if (last) {
               __syncwarp();
               if (lane == 0) mbar_arrive(aempty + p);
@@ -265,7 +279,7 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
           }
           // operand stage: (tile, parity) number c; stages of kZp parities, kZs of them in turn
           const uint32_t c = 2 * t + p, st = c / kZp, slot = st % kZs, use = st / kZs;
-          if (p % kZp == 0 && use > 0 && !wait_or_abort(zempty + slot, (use - 1) & 1, limit, abort, a.err)) return false;
+          if (p % kZp == 0 && use > 0 && !warp_wait_or_abort(zempty + slot, (use - 1) & 1, limit, abort, a.err)) return false;
           unsigned char *z = zl + (slot * kZp + p % kZp) * kZStage;
 #pragma unroll
           for (int e = 0; e < 4; ++e)
@@ -273,6 +287,14 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
             for (int k = 0; k < 2; ++k)  // row = correlation * 64 + block * 32 + lane
               *reinterpret_cast<uint4 *>(z + (e >> 1) * kOperand + (e & 1) * 1024 + k * 512) =
                   make_uint4(out[e][k][0], out[e][k][1], out[e][k][2], out[e][k][3]);
+          if constexpr (p == 0) {  // cos(pi f / 2) = (-1)^(f / 2): + on odd warps
+            const float sg = (warp & 1) ? 1.f : -1.f;
+            float *part = s_part + ((t & 1) * kContract + warp) * 128 + lane;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+              for (int e = 0; e < 2; ++e) part[e * 64 + k * 32] = sg * ee[k][e];
+          }
           if (p % kZp == kZp - 1) {
             fence_proxy_async();
             __syncwarp();
@@ -300,18 +322,18 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
       const int64_t rb = img * a.K * g.S + (row - img * g.S);
       for (int kt = k0; kt < k1; ++kt, ++t) {
         const uint32_t buf = t & 1, ph = (t >> 1) & 1;
-        if (!wait_or_abort(x0full + buf, ph, limit, abort, a.err) ||
-            !wait_or_abort(dfull + buf, ph, limit, abort, a.err)) {
+        if (!warp_wait_or_abort(x0full + buf, ph, limit, abort, a.err) ||
+            !warp_wait_or_abort(dfull + buf, ph, limit, abort, a.err)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const float x0 = s_x0[buf * 64 + (q & 1) * 32 + lane];
+        const float x0 = s_x0[buf * 64 + (q & 1) * 32 + lane], e64 = s_e[buf * 128 + q * 32 + lane];
         const int ref = kt * 8 + refl;
         const bool valid = row < a.rows && ref < a.K;
         const int64_t at = rb + static_cast<int64_t>(ref) * g.S;
         if (a.dbg_cc)
-          hybrid_debug_row(tmem + lanes + buf * 256, corr, x0, valid ? a.dbg_cc + at * 512 + corr * 256 : nullptr);
+          hybrid_debug_row(tmem + lanes + buf * 256, corr, x0, e64, valid ? a.dbg_cc + at * 512 + corr * 256 : nullptr);
         float best = -INFINITY;
         // 8 angles of each sum at a time; the loop is kept short (the roles
         // run different code at the same time and share the instruction
@@ -336,9 +358,9 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
             const float E = __uint_as_float(ee[j]), F = __uint_as_float(eo[j]);
             const float G = __uint_as_float(oe[j]), H = __uint_as_float(oo[j]);
             float v = (E + F) + fabsf(G + H), w = (E - F) + fabsf(G - H);
-            if (j == 0 && j0 == 0) {  // angles 0, 128; G, H are the sums of angles 64, 192
+            if (j == 0 && j0 == 0) {  // angles 0, 128; H is Oo at angle 64
               v = E + fabsf(F);
-              w = G + fabsf(H);
+              w = e64 + fabsf(H);
             }
             best = fmaxf(best, fmaxf(v, w));
           }
@@ -374,16 +396,12 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
               tc_fence_after();
               // core columns of 8 frequencies: 2048 bytes apart in an operand, 1024 in a matrix
               const uint64_t zr = umma_sdesc(zb + (slot * kZp + p % kZp) * kZStage, 2048, 128), zi = zr + (kOperand >> 4);
-              const uint64_t w0 = umma_sdesc(wb + (p ? 3 * kW : 0), 1024, 128), w1 = w0 + (kW >> 4),
-                             w2 = w1 + (kW >> 4);
+              const uint64_t w0 = umma_sdesc(wb + p * 2 * kW, 1024, 128), w1 = w0 + (kW >> 4);
 #pragma unroll
               for (int ks = 0; ks < 4; ++ks) {
                 umma_ss(dcol + p * 64, zr + ks * 256, w0 + ks * 128, idesc, ks > 0);        // Ee | Eo
                 umma_ss(dcol + 128 + p * 64, zi + ks * 256, w1 + ks * 128, idesc, ks > 0);  // Oe | Oo
               }
-              if (!p)
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) umma_ss(dcol + 128, zr + ks * 256, w2 + ks * 128, idesc, 1);  // Ee(64)
               if (p % kZp == kZp - 1) umma_commit(zempty + slot);
             }
             if (ok) umma_commit(dfull + buf);
@@ -412,7 +430,7 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
 #pragma unroll
           for (int j = 0; j < kHyb256N0; ++j) b[j] = load_frag(bp + j * 512);
           if (!kRegs && kt == k0) {
-            if (!wait_or_abort(afull, un & 1, limit, abort, a.err)) {
+            if (!warp_wait_or_abort(afull, un & 1, limit, abort, a.err)) {
               ok = false;
               break;
             }
@@ -421,7 +439,7 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(aempty);
           }
-          if (t >= 2 && !wait_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) {
+          if (t >= 2 && !warp_wait_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) {
             ok = false;
             break;
           }
@@ -433,8 +451,28 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
           }
           s_x0[buf * 64 + lane] = d0[0];
           s_x0[buf * 64 + 32 + lane] = d1[0];
-          __syncwarp();
-          if (lane == 0) mbar_arrive(x0full + buf);
+          // the parts of Ee(64): written with the even operands of the stage(s) of this tile
+#pragma unroll
+          for (int p = 0; p < 2 && ok; p += kZp) {
+            const uint32_t st = (2 * t + p) / kZp, slot = st % kZs;
+            ok = warp_wait_or_abort(zfull + slot, (st / kZs) & 1, limit, abort, a.err);
+            if (ok && p == 0) {
+              const float *part = s_part + buf * kContract * 128 + lane;
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                float e = 0.f;
+#pragma unroll
+                for (int w = 0; w < kContract; ++w) e += part[w * 128 + r * 32];
+                s_e[buf * 128 + r * 32 + lane] = e;
+              }
+            }
+            __syncwarp();
+            if (lane == 0) {
+              mbar_arrive(zempty + slot);
+              if (p == 0) mbar_arrive(x0full + buf);
+            }
+          }
+          if (!ok) break;
         }
       }
     } else if (warp == 14 && !kRegs) {
@@ -446,9 +484,10 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
       for (int64_t u = blockIdx.x; u < units && ok; u += gridDim.x, ++un) {
         const unsigned char *src = gA + static_cast<size_t>(u / splits) * kTile16;
         for (int p = 0; p < 2 && ok; ++p) {
-          if (un > 0 && !wait_or_abort(aempty + p, (un - 1) & 1, limit, abort, a.err)) ok = false;
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
+          if (un > 0 && !warp_wait_or_abort(aempty + p, (un - 1) & 1, limit, abort, a.err)) {
+            ok = false;
+            break;
+          }
           if (lane == 0) mbar_arrive_expect_tx(afull + p, (kContract * T + (p ? 0 : kHyb256N0)) * 512u);
           __syncwarp();
           fence_proxy_async();  // earlier reads of these fragments are done (aempty)

@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(u512::kThreads, 1)
             for (int i = 0; i < 16; ++i) out[2 + (i >> 3)][(i >> 2) & 1][i & 3] ^= 0x80008000u;
           }
           const uint32_t c = 2 * t + p;  // uses of the operand stage
-          if ((c > 0 && !wait_or_abort(zfree, (c - 1) & 1, limit, abort, a.err)) ||
-              (!p && t > 0 && !wait_or_abort(pfree, (t - 1) & 1, limit, abort, a.err))) {
+          if ((c > 0 && !warp_wait_or_abort(zfree, (c - 1) & 1, limit, abort, a.err)) ||
+              (!p && t > 0 && !warp_wait_or_abort(pfree, (t - 1) & 1, limit, abort, a.err))) {
             ok = false;
             break;
           }
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(u512::kThreads, 1)
       const int64_t rb = img * a.K * g.S + (row - img * g.S);
       for (int kt = k0; kt < k1; ++kt, ++t) {
         const uint32_t buf = t & 1;
-        if (!wait_or_abort(x0full + buf, (t >> 1) & 1, limit, abort, a.err) ||
-            !wait_or_abort(dfull, t & 1, limit, abort, a.err)) {
+        if (!warp_wait_or_abort(x0full + buf, (t >> 1) & 1, limit, abort, a.err) ||
+            !warp_wait_or_abort(dfull, t & 1, limit, abort, a.err)) {
           ok = false;
           break;
         }
@@ -356,8 +356,8 @@ __global__ void __launch_bounds__(u512::kThreads, 1)
             mma_frag<FP16>(d0, af, bf.x, bf.y);
             mma_frag<FP16>(d1, af, bf.z, bf.w);
           }
-          if ((t >= 2 && !wait_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) ||
-              !wait_or_abort(efull, t & 1, limit, abort, a.err)) {
+          if ((t >= 2 && !warp_wait_or_abort(dempty + buf, ((t >> 1) - 1) & 1, limit, abort, a.err)) ||
+              !warp_wait_or_abort(efull, t & 1, limit, abort, a.err)) {
             ok = false;
             break;
           }

@@ -348,16 +348,15 @@ const std::vector<uint32_t> &hybrid_matrices() {
     for (int m = 0; m < kMats; ++m)
       for (int j = 0; j < Q; ++j)
         for (int k = 0; k < Q; ++k) {
-          const bool odd = M == 256 ? m >= 3 : m == 2;
+          const bool odd = m >= 2;
           const int i = W * (k % 8) + k / 8, f = odd ? 2 * i + 1 : 2 * i + 2;
           double v = 0.0;
           if (M == 512) {
             v = m == 1 ? -sn(f * j) : c(f * j);                         // Ee, Oe, Eo
           } else {
-            if (m == 0 || m == 3) v = c(f * j);                         // Ee, Eo
+            if (m == 0 || m == 2) v = c(f * j);                         // Ee, Eo
             if (m == 1) v = -sn(f * j);                                 // Oe
-            if (m == 2) v = j == 0 ? c(f * Q) : 0.0;                    // X: Ee at angle M / 4
-            if (m == 4) v = j == 0 ? -sn(f * Q) : -sn(f * j);           // Oo; column 0: angle M / 4
+            if (m == 3) v = j == 0 ? -sn(f * Q) : -sn(f * j);           // Oo; column 0: angle M / 4
           }
           if (f == M / 2) v *= 0.5;                                     // its own mirror image
           const size_t byte = (static_cast<size_t>(m) * Q * Q + (k / 8) * (8 * Q) + (j / 8) * 64 + (j % 8) * 8 + k % 8) * 2;

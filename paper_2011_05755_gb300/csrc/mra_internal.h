@@ -77,7 +77,7 @@ struct Geometry {
   const int *chunk_f;     // [NCH + 1]
   // M = 256 kernel with the tcgen05 inverse DFT (null unless the handle uses
   // it; its k-steps are then ordered by contraction warp and parity): the
-  // five BF16 DFT matrices Ee, Oe, X, Eo, Oo (64 angles x 64 frequencies,
+  // four BF16 DFT matrices Ee, Oe, Eo, Oo (64 angles x 64 frequencies,
   // canonical K-major core matrices).
   // M = 512: the matrices Ee, Oe, Eo (128 x 128) and, per contraction warp,
   // {its first k-step, its k-steps, k-steps of the even, of the odd slots (4 bits each)}.
@@ -87,7 +87,7 @@ struct Geometry {
 };
 
 constexpr int kHyb256N0 = 3;    // k-steps of f = 0
-constexpr int kHyb256Mats = 5;
+constexpr int kHyb256Mats = 4;
 constexpr int kHyb512Mats = 3;
 
 constexpr int kTc256ChunkKs = 22;

@@ -109,6 +109,12 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, ui
   return false;
 }
 
+// The same by a whole warp, with one answer for all lanes.
+__device__ __forceinline__ bool warp_wait_or_abort(uint64_t *bar, uint32_t parity, uint32_t limit, volatile int *abort,
+                                                   int *err) {
+  return __all_sync(0xffffffffu, wait_or_abort(bar, parity, limit, abort, err));
+}
+
 // The same bounded wait by spinning instead of suspending, for the single
 // threads that issue TMA copies and MMAs (a suspended thread resumes later
 // than a spinning one sees the phase complete).  limit counts sleeps of the
