@@ -219,6 +219,20 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   }
   __syncthreads();
 
+  // Sample-table entries of the next pass over the samples, loaded while this
+  // one is sampled (and those of a group's first pass during the previous
+  // group's copy-out): 12,000 images of 76 px 16.77 -> 15.75 ms, 128 px 8.42 ->
+  // 8.25 ms; four or six entries a thread instead of eight: 16.3 ms.
+  constexpr int QU = 8;
+  float4 tn[QU];
+  auto load_taps = [&](int q0) {
+#pragma unroll
+    for (int u = 0; u < QU; ++u) {
+      const int q = q0 + u * NT;
+      tn[u] = q < NS ? __ldg(g.taps + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if constexpr (MODE == kPolarInt) load_taps(threadIdx.x);
   for (int s0 = blockIdx.x * R; s0 < a.rows_per_img; s0 += gridDim.x * R) {
     const int nrows = min(R, a.rows_per_img - s0);
     const int64_t row0 = img * a.rows_per_img + s0;
@@ -246,15 +260,12 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
           }
         }
       }
-      // eight samples per thread and pass, their tap loads issued together
-      constexpr int QU = 8;
+      // QU samples per thread and pass; the next pass's table entries load meanwhile
       for (int q0 = threadIdx.x; q0 < NS; q0 += QU * NT) {
         float4 tp[QU];
 #pragma unroll
-        for (int u = 0; u < QU; ++u) {
-          const int q = q0 + u * NT;
-          tp[u] = q < NS ? __ldg(g.taps + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        for (int u = 0; u < QU; ++u) tp[u] = tn[u];
+        if (q0 + QU * NT < NS) load_taps(q0 + QU * NT);
 #pragma unroll
         for (int u = 0; u < QU; ++u) {
           const int q = q0 + u * NT;
@@ -341,6 +352,7 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
                                                                     nrows, row0, warp, lane, fw);
     });
 
+    if constexpr (MODE == kPolarInt) load_taps(threadIdx.x);
     // Phase 3 (16-bit paths): copy-out in the layout of the tensor-core
     // kernel, 16 bytes per store.
     if constexpr (OUT != kOutF32) {
