@@ -23,7 +23,9 @@ constexpr int kRescoreThreads = 256;  // 8 warps per CTA (one image)
 // Registers are held to 64 per thread for M = 32..256, so that four CTAs
 // (images) fit on an SM where their shared memory allows (the 76-pixel
 // workload).
-template <int M>
+// PAIRS: ring transforms by warp_fft_pairs (M >= 256, and more candidates
+// than one to a CTA).
+template <int M, bool PAIRS>
 __global__ void __launch_bounds__(kRescoreThreads, (M >= 32 && M <= 256) ? 4 : 1)
     rescore_kernel(Geometry g, RescoreArgs a) {
   constexpr int T = IfftShape<M>::T;
@@ -111,7 +113,10 @@ __global__ void __launch_bounds__(kRescoreThreads, (M >= 32 && M <= 256) ? 4 : 1
       const int4 rd = s_rings[ring];
       const int N = rd.x, H = N >> 1;
       float2 *z = reinterpret_cast<float2 *>(samp + rd.y);
-      warp_fft_inplace(z, H, rd.w, M, twf, lane);
+      if constexpr (PAIRS)
+        warp_fft_pairs<M>(z, H, rd.w, twf, lane);
+      else
+        warp_fft_inplace(z, H, rd.w, M, twf, lane);
       __syncwarp();
       // in-place split: lane pair {kx, H - kx} reads and writes only its two slots
       const int wstep = M / N;
@@ -229,17 +234,16 @@ size_t rescore_smem(const Geometry &g) {
 
 // The kernel's dynamic shared-memory limit only ever grows (handles of
 // several geometries share the kernel).
-template <int M>
+template <int M, bool PAIRS>
 static cudaError_t rescore_smem_attr(size_t smem) {
   static size_t granted = 0;
-  return raise_smem_limit(rescore_kernel<M>, smem, granted);
+  return raise_smem_limit(rescore_kernel<M, PAIRS>, smem, granted);
 }
 
 template <int M>
 static cudaError_t launch_rescore_t(const Geometry &g, const RescoreArgs &a, cudaStream_t st) {
   const size_t smem = rescore_smem(g);
-  cudaError_t e = rescore_smem_attr<M>(smem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   // CTAs per image: as many (1, 2, 4, 8) as still run at once.  Each stages
   // the image again, so only calls that leave SMs idle are split (top-8 and
   // rescore together: one image of 64 px 131 -> 27 us, 200 images of 76 px 241
@@ -255,7 +259,16 @@ static cudaError_t launch_rescore_t(const Geometry &g, const RescoreArgs &a, cud
   const int64_t slots = static_cast<int64_t>(at_once) * (2 * smem + 2048 > 233472 ? 1 : (4 * smem + 4096 > 233472 ? 2 : 4));
   unsigned parts = 1;
   while (parts < kTopRows && a.n * parts * 2 <= slots) parts *= 2;
-  rescore_kernel<M><<<dim3(static_cast<unsigned>(a.n), parts), kRescoreThreads, smem, st>>>(g, a);
+  const dim3 grid(static_cast<unsigned>(a.n), parts);
+  if (M >= 256 && parts < kTopRows) {
+    e = rescore_smem_attr<M, (M >= 256)>(smem);
+    if (e != cudaSuccess) return e;
+    rescore_kernel<M, (M >= 256)><<<grid, kRescoreThreads, smem, st>>>(g, a);
+  } else {
+    e = rescore_smem_attr<M, false>(smem);
+    if (e != cudaSuccess) return e;
+    rescore_kernel<M, false><<<grid, kRescoreThreads, smem, st>>>(g, a);
+  }
   return cudaGetLastError();
 }
 
@@ -263,8 +276,8 @@ template <int M>
 static int rescore_occupancy_t(const Geometry &g) {
   const size_t smem = rescore_smem(g);
   int n = 0;
-  if (rescore_smem_attr<M>(smem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rescore_kernel<M>, kRescoreThreads, smem) != cudaSuccess) {
+  if (rescore_smem_attr<M, (M >= 256)>(smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rescore_kernel<M, (M >= 256)>, kRescoreThreads, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

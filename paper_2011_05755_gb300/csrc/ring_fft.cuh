@@ -79,6 +79,97 @@ __device__ __forceinline__ void warp_fft_inplace(float2 *z, int H, int logH, int
   }
 }
 
+// The same transform, natural order in and out, with two stages per pass over
+// the shared memory: each lane holds four values in registers, the bit reversal
+// is in the first pass's loads, and every butterfly is the one above, so the
+// result has the same bits.  Between passes value i sits at
+// i ^ (((i >> 4) & 3) << 2), which spreads the strided passes over the banks; the
+// last pass writes natural order.  It halves the shared-memory traffic of the
+// transform but leaves most lanes idle on rings of 64 samples and fewer: the
+// rescore of 12,000 images of 76 px (M = 256) takes 5.06 -> 4.60 ms, of 600
+// images of 128 px (M = 512) 1.72 -> 1.51 ms, of 5,003 images of 32 px
+// (M = 128) 0.44 -> 0.52 ms, hence M >= 256 only.  Where each candidate has a
+// CTA of its own (a few images), the shorter chain of the plain transform is
+// faster instead (one image of 64 px: 46 against 49 us for the whole call).  Not inlined: inlined, its
+// addresses are kept across the candidates and spill (4.71 ms).
+__device__ __forceinline__ int fft_swz(int i) { return i ^ (((i >> 4) & 3) << 2); }
+
+__device__ __forceinline__ void butterfly(float2 &u, float2 &v, float2 w) {
+  const float2 t = cmul(w, v);
+  v = csub(u, t);
+  u = cadd(u, t);
+}
+
+template <int M>
+__device__ __noinline__ void warp_fft_pairs(float2 *z, int H, int logH, const float2 *fwd_tw, int lane) {
+  constexpr int PER = M >= 512 ? M / 256 : 1;  // groups of four per lane: H <= M / 2
+  const int G = H >> 2;
+  const int brs = 34 - logH;  // bit reversal of logH - 2 bits
+#pragma unroll 1
+  for (int st = 0; st + 2 <= logH; st += 2) {  // stages h = 2^st and 2 h
+    const int h = 1 << st;
+    const bool last = st + 2 == logH;
+    float2 x[PER][4];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int gi = lane + 32 * i;
+      if (gi < G) {
+        const int p = gi & (h - 1), base = (gi - p) * 4 + p;
+        if (st == 0) {  // value 4 gi + e comes from its bit-reversed place
+          const int rg = logH > 2 ? static_cast<int>(__brev(static_cast<unsigned>(gi)) >> brs) : 0;
+          x[i][0] = z[rg];
+          x[i][1] = z[rg + (H >> 1)];
+          x[i][2] = z[rg + G];
+          x[i][3] = z[rg + 3 * G];
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[i][e] = z[fft_swz(base + e * h)];
+        }
+        const int step = M >> (st + 2);
+        const float2 w1 = fwd_tw[2 * p * step];
+        butterfly(x[i][0], x[i][1], w1);
+        butterfly(x[i][2], x[i][3], w1);
+        butterfly(x[i][0], x[i][2], fwd_tw[p * step]);
+        butterfly(x[i][1], x[i][3], fwd_tw[(p + h) * step]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int gi = lane + 32 * i;
+      if (gi < G) {
+        const int p = gi & (h - 1), base = (gi - p) * 4 + p;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) z[last ? base + e * h : fft_swz(base + e * h)] = x[i][e];
+      }
+    }
+    __syncwarp();
+  }
+  if (logH & 1) {
+    const int h = H >> 1, step = M >> logH;
+    float2 x[2 * PER][2];
+#pragma unroll
+    for (int i = 0; i < 2 * PER; ++i) {
+      const int p = lane + 32 * i;
+      if (p < h) {
+        x[i][0] = z[fft_swz(p)];
+        x[i][1] = z[fft_swz(p + h)];
+        butterfly(x[i][0], x[i][1], fwd_tw[p * step]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 2 * PER; ++i) {
+      const int p = lane + 32 * i;
+      if (p < h) {
+        z[p] = x[i][0];
+        z[p + h] = x[i][1];
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // Forward FFT of H complex points (power of two, 4..256) held in shared
 // memory, by a group of T threads of one warp (T = H / 16 for H >= 32, else
 // one thread): thread t transforms z(t + T a), a = 0..U-1, in registers,
