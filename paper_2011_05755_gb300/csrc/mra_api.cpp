@@ -746,8 +746,8 @@ int ensure_chunk_workspace(mra_handle *h) {
       // the default chunk in whole waves of the FP32 rescore (one CTA per
       // image) when that costs at most a tenth of it: a chunk that ends with
       // a nearly empty wave leaves most SMs idle for one rescore CTA's time
-      // (the polar kernel's waves, four CTAs per image at two per SM, divide
-      // the same count at L = 76)
+      // (the polar kernel's waves, one CTA per image and SM, divide the same
+      // count)
       int dev = 0, sms = 0;
       const int occ = mra::rescore_ctas_per_sm(h->g);
       if (occ > 0 && cudaGetDevice(&dev) == cudaSuccess &&
