@@ -445,9 +445,11 @@ inline int polar_cta_rows(const Geometry &g, int mode, bool out16) {
 // the 76-, 90- and 128-pixel workloads: 12,000 images of 76 px, 81 shifts,
 // 16-bit output: R = 2 28.4 ms, 3 23.8, 4 20.0, 5 19.0, and 21.4 for two CTAs
 // of 8 warps with 2 rows each; 5,003 images of 32 px on a half-pixel grid of
-// 49: 4 rows 1.92 ms, 6 1.47, 8 1.35, two small CTAs with 4 rows each 1.77), so large groups win on long stacks, where they
-// also share table entries and pixel columns, and one row per CTA on calls
-// whose rows do not fill the SMs.
+// 49: 4 rows 1.92 ms, 6 1.47, 8 1.35, two small CTAs with 4 rows each 1.77), so
+// large groups win on long stacks, where they also share table entries and
+// pixel columns, and one row per CTA on calls whose rows do not fill the SMs.
+// (With the warp count and table loads as they are now: 5 rows 15.8 ms, 8 rows
+// of 32 px 1.16 ms; bound by the shared-memory data pipe, 81 % of its peak.)
 inline int polar_bordered_rows(const PolarArgs &a, int most, int sms) {
   int best = 1;
   double best_cost = 1e300;
