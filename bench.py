@@ -391,7 +391,7 @@ def main():
             cc_line = {"bound": "alu", "kernel": kname + " (FP32 contraction + inverse angular DFT + argmax)",
                        "achieved": flops / cc_s / 1e12, "peak": alu_peak, "unit": "TFLOP/s", "peak_source": alu_src}
         else:
-            kname = {256: "cc_hybrid256_kernel", 512: "cc_hybrid512_kernel"}.get(info["M"], "cc_tc_kernel")
+            kname = {256: "cc_hybrid256_kernel", 512: "cc_tc512_kernel"}.get(info["M"], "cc_tc_kernel")
             if info["M"] == 256 and choice["kernel"] == mra.MRA_KERNEL_MMA_SYNC:
                 kname = "cc_tc256_kernel"
             tc_idft = info["M"] in (256, 512)  # the inverse DFT on tensor cores too (M <= 128: FP32)

@@ -13,11 +13,11 @@
 // (p rows) for 8 rows x 4 references.  A tile of 8 rows x 8 references is
 // two such MMAs per k-step.  Operands are BF16 (or FP16), accumulation FP32.
 //
-// For M = 256 (rings up to 40) the per-pair angular state is kept as BF16 in
-// shared memory and the inverse angular DFT runs on tensor cores too
-// (cc_tc256_kernel, for MRA_KERNEL_MMA_SYNC: the default kernel is that of
-// k_umma256.cu); for M <= 128 the state stays FP32 (cc_tc_kernel); M = 512 is
-// in k_umma512.cu.  Either way the row maxima select the 8 rows
+// For M = 256 (rings up to 40) and M = 512 the per-pair angular state is kept
+// as BF16 in shared memory and the inverse angular DFT runs on tensor cores
+// too (cc_tc256_kernel, cc_tc512_kernel); for M <= 128 the state stays FP32
+// (cc_tc_kernel).  (The default at M = 256 is the kernel of k_umma256.cu;
+// cc_tc256_kernel serves MRA_KERNEL_MMA_SYNC.)  Either way the row maxima select the 8 rows
 // (reference, shift, mirror) per image that the rescore kernel recomputes
 // from scratch in FP32; its argmax is the answer.
 #include <cuda_bf16.h>
@@ -453,6 +453,231 @@ __global__ void __launch_bounds__(kTc256Threads, 2) cc_tc256_kernel(Geometry g, 
   }
 }
 
+// M = 512 kernel (rings up to 81): the tile walk and chunked staging of the
+// M = 256 kernel with one CTA of 16 warps per SM (the BF16 spectra of the
+// 64 pairs take 128 KB) and chunks of up to kTc512ChunkKs k-steps.
+// Spectrum word of Z(f) in a pair's 512-word buffer: z512_fold(f) ^ s with
+// s = 4 (pair / 8) + (pair % 4) < 32, so the contraction's stores (32 lanes,
+// 32 pairs, one f) hit distinct banks.  Phase 2: the inverse DFT on tensor
+// cores by an even / odd split (decimation in frequency index):
+//     c(n)       = E(n) + w512^n O(n),    c(n + 256) = E(n) - w512^n O(n),
+//     E(n) = sum_m Z(2 m) w256^(m n),     O(n) = sum_m Z(2 m + 1) w256^(m n),
+// n = 0..255: two 256-point inverse DFTs per pair (idft256_core) and a
+// radix-2 combine in FP32, one warp per pair.  z512_fold places the words
+// those 256-point DFTs load (f = 2 (8 nb + g + 16 a) (+1)) in 32 distinct
+// banks for every load of the warp.
+//
+// Contraction stage: 600 images of 128 px, K = 200, 169 shifts 38.3 ms; 1,500
+// of 96 px, K = 200, 49 shifts 22.7 ms (whole calls 48.2 and 27.3 ms).  The
+// scheme of k_umma256.cu at this length took 20.6 and 11.8 ms, but its table is
+// rounded at other places: of 924,000 images 23 got another pose (the row with
+// the largest FP32 coefficient is then not among this table's eight; all 23
+// were closer to the FP32 path there), and poses must not change with the kernel.
+__device__ __forceinline__ int z512_fold(int f) { return f ^ ((f >> 6) & 1) ^ (((f >> 7) & 1) << 4); }
+
+constexpr int kTc512Warps = 16;
+constexpr int kTc512Threads = 32 * kTc512Warps;
+constexpr int kTc512MaxChunks = 48;
+constexpr size_t kTc512Stage = static_cast<size_t>(kTc512ChunkKs) * 1024;
+constexpr size_t kTc512Smem = 2 * kTc512Stage + 64 * 512 * sizeof(uint32_t) + 2 * sizeof(uint64_t) + 8 * sizeof(int2) +
+                              (258 + kTc512MaxChunks + 2) * sizeof(int);
+static_assert(kTc512Smem <= 232448, "M = 512 kernel exceeds 227 KB of shared memory");
+
+template <bool FP16>
+__global__ void __launch_bounds__(kTc512Threads, 1) cc_tc512_kernel(Geometry g, TcArgs a, int ref_tiles) {
+  constexpr int M = 512, PAIRS = 64, NF = M / 2 + 1;
+  extern __shared__ float4 smem_f4[];
+  unsigned char *stage = reinterpret_cast<unsigned char *>(smem_f4);
+  uint32_t *Zw = reinterpret_cast<uint32_t *>(stage + 2 * kTc512Stage);  // [64 pairs][512 words]
+  uint64_t *full = reinterpret_cast<uint64_t *>(Zw + PAIRS * M);
+  int2 *rinfo = reinterpret_cast<int2 *>(full + 2);  // {image, shift} of the tile's rows
+  int *s_kso = reinterpret_cast<int *>(rinfo + 8);   // [NF + 1]
+  int *s_cf = s_kso + NF + 1;                        // [NCH + 1]
+
+  const int64_t rt = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nch = g.NCH;
+  const int total = ref_tiles * nch;
+  for (int i = tid; i <= NF; i += kTc512Threads) s_kso[i] = g.kso[i];
+  for (int i = tid; i <= nch; i += kTc512Threads) s_cf[i] = g.chunk_f[i];
+  if (tid < 8) {
+    const int64_t row = rt * 8 + tid;
+    const int img = static_cast<int>(static_cast<uint32_t>(row) / static_cast<uint32_t>(g.S));  // rows < 2^31
+    rinfo[tid] = make_int2(img, static_cast<int>(row - static_cast<int64_t>(img) * g.S));
+  }
+  if (tid == 0) {
+    mbar_init(full, 1);
+    mbar_init(full + 1, 1);
+  }
+  mbar_init_fence();
+  __syncthreads();
+
+  auto issue = [&](int q) {  // thread 0: stage chunk q % nch of reference tile q / nch into buffer q & 1
+    const int kt = q / nch, c = q - kt * nch;
+    const int k0 = s_kso[s_cf[c]];
+    const uint32_t nks = static_cast<uint32_t>(s_kso[s_cf[c + 1]] - k0);
+    unsigned char *dst = stage + (q & 1) * kTc512Stage;
+    fence_proxy_async();
+    mbar_arrive_expect_tx(full + (q & 1), nks * 1024u);
+    bulk_g2s(dst, a.A16 + (rt * g.KS + k0) * 32, nks * 512u, full + (q & 1));
+    bulk_g2s(dst + nks * 512u, a.B16 + (static_cast<int64_t>(kt) * g.KS + k0) * 32, nks * 512u, full + (q & 1));
+  };
+  if (tid == 0) {
+    issue(0);
+    if (total > 1) issue(1);
+  }
+
+  const int g8 = lane >> 2, t4 = lane & 3;
+  const int sw = 4 * g8 + t4;              // spectrum swizzle of both of this lane's phase-1 pairs
+  uint32_t *z0 = Zw + (8 * g8 + t4) * M;   // pair (row g8, reference t4)
+  uint32_t *z1 = z0 + 4 * M;               // pair (row g8, reference 4 + t4)
+  const int S = g.S;
+
+  // lane constants of phase 2: the 16-point DFT fragments, the folded word
+  // positions of the even spectrum words this lane loads (the odd word of
+  // each sits at the position XOR 1), the 256-point stage twiddles
+  // w256^(t k) = w512^(2 t k) and the combine twiddles w512^n of its angles
+  // (g.angles[q] = exp(2 pi i q / M))
+  uint32_t a1[16], b2[16];
+  {
+    const uint4 *fa = reinterpret_cast<const uint4 *>(g.dft16) + lane * 4;
+    const uint4 *fb = reinterpret_cast<const uint4 *>(g.dft16 + 512) + lane * 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint4 va = __ldg(fa + i), vb = __ldg(fb + i);
+      a1[4 * i] = va.x;
+      a1[4 * i + 1] = va.y;
+      a1[4 * i + 2] = va.z;
+      a1[4 * i + 3] = va.w;
+      b2[4 * i] = vb.x;
+      b2[4 * i + 1] = vb.y;
+      b2[4 * i + 2] = vb.z;
+      b2[4 * i + 3] = vb.w;
+    }
+  }
+  int zoff[8];
+  float2 tws[8], wn[8];
+  {
+    const int aa[4] = {2 * t4, 2 * t4 + 1, 2 * t4 + 8, 2 * t4 + 9};
+#pragma unroll
+    for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zoff[nb * 4 + e] = z512_fold(2 * (8 * nb + g8 + 16 * aa[e]));
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int k = g8 + 8 * (q >> 1);
+        tws[b * 4 + q] = __ldg(g.angles + ((2 * (8 * b + 2 * t4 + (q & 1)) * k) & (M - 1)));
+        wn[b * 4 + q] = __ldg(g.angles + k + 16 * (8 * b + 2 * t4 + (q & 1)));
+      }
+  }
+
+  int q = 0;  // global chunk index
+  for (int kt = 0; kt < ref_tiles; ++kt) {
+    // ---------------- Phase 1: tensor-core contraction ----------------
+    for (int c = 0; c < nch; ++c, ++q) {
+      const int buf = q & 1;
+      const bool ok = mbar_wait_bounded(full + buf, static_cast<uint32_t>((q >> 1) & 1),
+                                        q == 0 ? a.first_wait_limit : a.wait_limit);
+      if (ok) {
+        const int f0 = s_cf[c], f1 = s_cf[c + 1];
+        const int kbase = s_kso[f0];
+        const int nks_c = s_kso[f1] - kbase;
+        const uint4 *stA = reinterpret_cast<const uint4 *>(stage + buf * kTc512Stage) + lane;
+        const uint4 *stB = stA + nks_c * 32;
+        for (int f = f0 + warp; f < f1; f += kTc512Warps) {
+          const int jb = s_kso[f] - kbase, nj = s_kso[f + 1] - s_kso[f];  // 1..6 k-steps
+          float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int jj = 0; jj < kTc512MaxKsPerF; ++jj) {
+            if (jj < nj) {
+              const int j = (jb + jj) * 32;
+              const uint4 af = stA[j], bf = stB[j];
+              mma16816<FP16>(d0, af, make_uint2(bf.x, bf.y));
+              mma16816<FP16>(d1, af, make_uint2(bf.z, bf.w));
+            }
+          }
+          // lane (g8, t4): d[0..1] = Re/Im Z(f), d[2..3] = Im/Re Z(M - f)
+          const int pf = z512_fold(f) ^ sw;
+          z0[pf] = pack_bf2(d0[0], d0[1]);
+          z1[pf] = pack_bf2(d1[0], d1[1]);
+          if (f != 0 && f != M / 2) {
+            const int pm = z512_fold(M - f) ^ sw;
+            z0[pm] = pack_bf2(d0[3], d0[2]);
+            z1[pm] = pack_bf2(d1[3], d1[2]);
+          }
+        }
+      }
+      if (__syncthreads_or(!ok)) {  // uniform: every thread leaves
+        if (tid == 0) {
+          atomicOr(a.err, 1);
+          // let the copies still in flight land before the CTA's memory goes
+          mbar_wait_bounded(full + (q & 1), static_cast<uint32_t>((q >> 1) & 1), a.wait_limit);
+          if (q + 1 < total)
+            mbar_wait_bounded(full + ((q + 1) & 1), static_cast<uint32_t>(((q + 1) >> 1) & 1), a.wait_limit);
+        }
+        return;
+      }
+      if (tid == 0 && q + 2 < total) issue(q + 2);
+    }
+
+    // ---------------- Phase 2: tensor-core inverse DFT (even / odd split), row maxima ----------------
+    // warp w: reference w % 8 of the tile, rows 4 (w / 8) .. 4 (w / 8) + 3
+    const int refl = warp & 7;
+    const int ref = kt * 8 + refl;
+    const int i0 = 4 * (warp >> 3);
+    const int64_t left = a.rows - rt * 8 - i0;
+    const int nvalid = ref < a.K ? (left >= 4 ? 4 : (left > 0 ? static_cast<int>(left) : 0)) : 0;
+#pragma unroll 1
+    for (int r = 0; r < nvalid; ++r) {  // padding pairs are skipped (warp-uniform)
+      const int i = i0 + r, pc = 8 * i + refl;
+      const uint32_t *zp = Zw + pc * M;
+      const int swp = 4 * (pc >> 3) + (pc & 3);
+      float de[4][4], dd[4][4];  // E and O at this lane's angles (idft256_core's fragment order)
+      {
+        uint32_t z[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z[e] = zp[zoff[e] ^ swp];
+        idft256_core(z, tws, a1, b2, de);
+      }
+      {
+        uint32_t z[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z[e] = zp[zoff[e] ^ 1 ^ swp];
+        idft256_core(z, tws, a1, b2, dd);
+      }
+      const int2 ri = rinfo[i];
+      const int64_t rbase = (static_cast<int64_t>(ri.x) * a.K + ref) * S + ri.y;
+      float *dbg = a.dbg_cc ? a.dbg_cc + rbase * 2 * M : nullptr;
+      float vu = -INFINITY, vm = -INFINITY;
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 w = wn[b * 4 + q];
+          const float orr = dd[b][q], oi = dd[b + 2][q];
+          const float wr = fmaf(w.x, orr, -w.y * oi), wi = fmaf(w.x, oi, w.y * orr);
+          const float c1r = de[b][q] + wr, c1i = de[b + 2][q] + wi;  // angle n
+          const float c2r = de[b][q] - wr, c2i = de[b + 2][q] - wi;  // angle n + 256
+          vu = fmaxf(vu, fmaxf(c1r, c2r));
+          vm = fmaxf(vm, fmaxf(c1i, c2i));
+          if (dbg) {
+            const int n = g8 + 8 * (q >> 1) + 16 * (8 * b + 2 * t4 + (q & 1));
+            dbg[n] = c1r;
+            dbg[n + 256] = c2r;
+            dbg[M + n + 256] = c1i;  // Im c(n) at (n + M / 2) mod M
+            dbg[M + n] = c2i;        // Im c(n + 256) at n
+          }
+        }
+      // (reducing two pairs together as the M = 256 kernel does needs registers this kernel does not have)
+      const float best = warp_max2(vu, vm, lane);
+      if ((lane & 15) == 0) a.rowmax[rbase * 2 + (lane >> 4)] = (lane && !g.mirror) ? -INFINITY : best;
+    }
+    __syncthreads();  // the next tile's contraction overwrites the pair buffers
+  }
+}
+
 template <int M, int KT, bool FP16>
 __global__ void __launch_bounds__(TcShape<M, KT>::THREADS) cc_tc_kernel(Geometry g, TcArgs a) {
   using Sh = TcShape<M, KT>;
@@ -722,8 +947,26 @@ static cudaError_t launch_tc256(const Geometry &g, const TcArgs &a, cudaStream_t
   return cudaGetLastError();
 }
 
+template <bool FP16>
+static cudaError_t launch_tc512(const Geometry &g, const TcArgs &a, cudaStream_t st) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(cc_tc512_kernel<FP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kTc512Smem));
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
+  if (row_tiles <= 0) return cudaSuccess;
+  if (g.NCH > kTc512MaxChunks) return cudaErrorInvalidValue;
+  cc_tc512_kernel<FP16><<<static_cast<unsigned>(row_tiles), kTc512Threads, kTc512Smem, st>>>(
+      g, a, (a.K + kTile - 1) / kTile);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_cc_tc(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st) {
   if (g.M == 256) return fp16 ? launch_tc256<true>(g, a, st) : launch_tc256<false>(g, a, st);
+  if (g.M == 512) return fp16 ? launch_tc512<true>(g, a, st) : launch_tc512<false>(g, a, st);
 #define MRA_TC_CASE(MM, KK) \
   case MM: return fp16 ? launch_tc_t<MM, KK, true>(g, a, st) : launch_tc_t<MM, KK, false>(g, a, st);
   switch (g.M) {

@@ -73,9 +73,11 @@
 // the device error flag, every role leaves its loop, the copying lane waits
 // for its copies in flight, the issuer for its MMAs, and the TMEM is
 // released.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
 #include "../../include/mra.h"
 #include "dev_util.cuh"
-#include "hybrid.cuh"
 #include "mra_internal.h"
 #include "smem_limit.cuh"
 #include "umma.cuh"
@@ -98,6 +100,31 @@ constexpr uint32_t kMisc = kWBytes + 2 * (64 + 128 + kContract * 128) * 4 + kNum
 __host__ __device__ constexpr int z_parities(int pattern) { return pattern == 0 ? 2 : 1; }
 __host__ __device__ constexpr int z_stages(int pattern) { return pattern == 0 ? 2 : 1; }
 }  // namespace u256
+
+template <bool FP16>
+__device__ __forceinline__ void mma_frag(float (&d)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
+  if constexpr (FP16)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ uint32_t pack_bf2u(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+__device__ __forceinline__ uint4 load_frag(const unsigned char *p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
 
 // The k-steps of the 8 slots of a warp and parity (fewer are padded with
 // zero fragments): pattern 0 = {3,2,2,2,1,1,1,1}, 1 = {3,3,2,2,2,2,2,2}.
@@ -133,8 +160,7 @@ __device__ __forceinline__ void contract_parity(FA &&fa, FB &&fb, Done &&done, u
     });
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      float v[4];
-      pair_sums(d[k], v);
+      const float v[4] = {d[k][0] + d[k][3], d[k][1] + d[k][2], d[k][1] - d[k][2], d[k][3] - d[k][0]};
       if constexpr (SUM) {
 #pragma unroll
         for (int e = 0; e < 2; ++e)
@@ -506,6 +532,27 @@ __global__ void __launch_bounds__(u256::kThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 12) tmem_dealloc(tmem, 512);
+}
+
+// Units of work are (row tile, range of reference tiles): `splits` ranges
+// per row tile, chosen to minimise the time of the fullest SM,
+// waves x (tiles per unit + the unit's load of its row fragments, about one
+// tile).  One range when the row tiles fill many waves (each row tile's
+// fragments are then loaded once); more when the stack is so small that
+// whole row tiles would leave SMs idle.
+static int pick_splits(int64_t row_tiles, int ref_tiles, int sms) {
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int s = 1; s <= ref_tiles; ++s) {
+    const int per = (ref_tiles + s - 1) / s;
+    if ((ref_tiles + per - 1) / per != s) continue;  // ranges must not be empty
+    const int64_t cost = (row_tiles * s + sms - 1) / sms * (per + 1);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return best;
 }
 
 template <int PATTERN, bool FP16>

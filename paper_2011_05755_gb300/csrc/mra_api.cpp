@@ -330,36 +330,29 @@ uint16_t bf16_bits(double v) {  // round to nearest even (|v| <= 1)
   return static_cast<uint16_t>((u + 0x7fffu + ((u >> 16) & 1u)) >> 16);
 }
 
-// BF16 DFT matrices of the kernels with the tcgen05 inverse DFT, M / 4 angles
-// x M / 4 frequencies each, in canonical K-major core matrices.  With W
-// contraction warps, K index 8 w + s is frequency number W s + w of its
-// parity; as the rings that reach a frequency never grow in number with it,
-// the frequencies sorted by k-step count are in ascending order whatever the
-// rings, and the matrices are the same for every handle of an M.
-template <int M>
+// BF16 DFT matrices of the M = 256 kernel with the tcgen05 inverse DFT (four
+// of 64 angles x 64 frequencies, canonical K-major core matrices).  K index
+// 8 w + s is frequency number 8 s + w of its parity; as the rings that reach a
+// frequency never grow in number with it, the frequencies sorted by k-step
+// count are in ascending order whatever the rings, and the matrices are the
+// same for every handle.
 const std::vector<uint32_t> &hybrid_matrices() {
   static const std::vector<uint32_t> mats = [] {
-    constexpr int Q = M / 4, W = Q / 8, kMats = M == 256 ? mra::kHyb256Mats : mra::kHyb512Mats;
-    std::vector<double> cosine(M);
-    for (int i = 0; i < M; ++i) cosine[i] = std::cos(kTwoPi * i / M);
-    auto c = [&](int i) { return cosine[((i % M) + M) % M]; };
-    auto sn = [&](int i) { return c(i - M / 4); };
-    std::vector<uint32_t> wm(static_cast<size_t>(kMats) * Q * Q / 2, 0);
-    for (int m = 0; m < kMats; ++m)
-      for (int j = 0; j < Q; ++j)
-        for (int k = 0; k < Q; ++k) {
-          const bool odd = m >= 2;
-          const int i = W * (k % 8) + k / 8, f = odd ? 2 * i + 1 : 2 * i + 2;
+    std::vector<double> cosine(256);
+    for (int i = 0; i < 256; ++i) cosine[i] = std::cos(kTwoPi * i / 256);
+    auto c = [&](int i) { return cosine[((i % 256) + 256) % 256]; };
+    auto sn = [&](int i) { return c(i - 64); };
+    std::vector<uint32_t> wm(mra::kHyb256Mats * 2048, 0);
+    for (int m = 0; m < mra::kHyb256Mats; ++m)
+      for (int j = 0; j < 64; ++j)
+        for (int k = 0; k < 64; ++k) {
+          const int i = 8 * (k % 8) + k / 8, f = m >= 2 ? 2 * i + 1 : 2 * i + 2;
           double v = 0.0;
-          if (M == 512) {
-            v = m == 1 ? -sn(f * j) : c(f * j);                         // Ee, Oe, Eo
-          } else {
-            if (m == 0 || m == 2) v = c(f * j);                         // Ee, Eo
-            if (m == 1) v = -sn(f * j);                                 // Oe
-            if (m == 3) v = j == 0 ? -sn(f * Q) : -sn(f * j);           // Oo; column 0: angle M / 4
-          }
-          if (f == M / 2) v *= 0.5;                                     // its own mirror image
-          const size_t byte = (static_cast<size_t>(m) * Q * Q + (k / 8) * (8 * Q) + (j / 8) * 64 + (j % 8) * 8 + k % 8) * 2;
+          if (m == 0 || m == 2) v = c(f * j);                           // Ee, Eo
+          if (m == 1) v = -sn(f * j);                                   // Oe
+          if (m == 3) v = j == 0 ? -sn(f * 64) : -sn(f * j);            // Oo; column 0: angle 64
+          if (f == 128) v *= 0.5;                                       // its own mirror image
+          const size_t byte = static_cast<size_t>(m) * 8192 + (k / 8) * 1024 + (j / 8) * 128 + (j % 8) * 16 + (k % 8) * 2;
           wm[byte / 4] |= static_cast<uint32_t>(bf16_bits(v)) << (byte % 4 * 8);
         }
     return wm;
@@ -464,30 +457,6 @@ int build_tables(mra_handle *h) {
       kso = pos;
       ksinfo = info;
     }
-  }
-  // M = 512 kernel: f = 0 first, then per contraction warp w its even
-  // frequencies 2 (16 s + w) + 2 and its odd ones 2 (16 s + w) + 1, s = 0..7.
-  std::vector<int4> sched;
-  if (M == 512 && h->half) {
-    std::vector<int2> info;
-    std::vector<int> pos(H + 2, 0);
-    auto place = [&](int f) {
-      const int n = kso[f + 1] - kso[f];
-      pos[f] = static_cast<int>(info.size());
-      for (int j = 0; j < n; ++j) info.push_back(make_int2(f, j));
-      return n;
-    };
-    place(0);
-    for (int w = 0; w < 16; ++w) {
-      int4 s = make_int4(static_cast<int>(info.size()), 0, 0, 0);
-      for (int p = 0; p < 2; ++p)
-        for (int sl = 0; sl < 8; ++sl) (p ? s.w : s.z) |= place(2 * (16 * sl + w) + 2 - p) << (4 * sl);
-      s.y = static_cast<int>(info.size()) - s.x;
-      sched.push_back(s);
-    }
-    pos[H + 1] = static_cast<int>(info.size());
-    kso = pos;
-    ksinfo = info;
   }
   std::vector<int> binpos16(NBIN);
   std::vector<int> binpos(NBIN);
@@ -640,11 +609,16 @@ int build_tables(mra_handle *h) {
     if ((rc = upload(h, kpos, &g.kpos, "frequency bases"))) return rc;
     if ((rc = upload(h, kpos16, &g.kpos16, "16-bit frequency bases"))) return rc;
   }
-  if (M == 256 && h->half && pattern < 0) {
-    // whole frequencies per staging chunk of the MRA_KERNEL_MMA_SYNC kernel, greedily
+  if (h->half && pattern < 0 && M >= 256) {
+    // whole frequencies per staging chunk of the MRA_KERNEL_MMA_SYNC (M = 256) and M = 512 kernels, greedily
+    const int cap = g.M == 512 ? mra::kTc512ChunkKs : mra::kTc256ChunkKs;
     std::vector<int> chunk_f(1, 0);
-    for (int f = 0; f <= H; ++f)
-      if (f > chunk_f.back() && kso[f + 1] - kso[chunk_f.back()] > mra::kTc256ChunkKs) chunk_f.push_back(f);
+    for (int f = 0; f <= H; ++f) {
+      const int start = kso[chunk_f.back()];
+      if (f > chunk_f.back() && kso[f + 1] - start > cap) chunk_f.push_back(f);
+      if (g.M == 512 && kso[f + 1] - kso[f] > mra::kTc512MaxKsPerF)
+        return set_err(h, MRA_EINVAL, "more than %d k-steps at frequency %d", mra::kTc512MaxKsPerF, f);
+    }
     chunk_f.push_back(H + 1);
     g.NCH = static_cast<int>(chunk_f.size()) - 1;
     if ((rc = upload(h, chunk_f, &g.chunk_f, "staging chunks"))) return rc;
@@ -689,12 +663,8 @@ int build_tables(mra_handle *h) {
     if ((rc = upload(h, frag, &g.dft16, "DFT fragments"))) return rc;
   }
   if (pattern >= 0) {
-    if ((rc = upload(h, hybrid_matrices<256>(), &g.hyb_w, "inverse-DFT matrices"))) return rc;
+    if ((rc = upload(h, hybrid_matrices(), &g.hyb_w, "inverse-DFT matrices"))) return rc;
     g.hyb_pattern = pattern;
-  }
-  if (!sched.empty()) {
-    if ((rc = upload(h, hybrid_matrices<512>(), &g.hyb_w, "inverse-DFT matrices"))) return rc;
-    if ((rc = upload(h, sched, &g.hyb_sched, "contraction schedule"))) return rc;
   }
   if ((rc = dev_alloc(h, &h->d_err, sizeof(int), "failure flags"))) return rc;
   h->tables.push_back(h->d_err);
@@ -953,9 +923,7 @@ int align_chunk_half(mra_handle *h, const float *imgs, int64_t cnt, mra_pose_t *
   t.first_wait_limit = first_wait_limit();
   int rec = prof_begin(h, MRA_STAGE_CC, st);
   if (h->g.hyb_w) {
-    rc = check_launch(h, h->g.M == 256 ? mra::launch_cc_hybrid256(h->g, t, h->fp16, st)
-                                       : mra::launch_cc_hybrid512(h->g, t, h->fp16, st),
-                      "tcgen05 contraction/IFFT kernel");
+    rc = check_launch(h, mra::launch_cc_hybrid256(h->g, t, h->fp16, st), "tcgen05 contraction/IFFT kernel");
   } else {
     rc = check_launch(h, mra::launch_cc_tc(h->g, t, h->fp16, st), "tensor-core contraction/IFFT kernel");
   }

@@ -71,26 +71,25 @@ struct Geometry {
   // inverse angular DFT (M = 256): [0, 512) stage-1 A, [512, 1024) stage-2 B,
   // each [32 lanes][16 words].
   const uint32_t *dft16;
-  // Staging chunks of the M = 256 mma.sync kernel: chunk c holds the whole
-  // frequencies [chunk_f[c], chunk_f[c + 1]), at most kTc256ChunkKs k-steps.
+  // Staging chunks of the M = 256 and M = 512 tensor-core kernels: chunk c
+  // holds the whole frequencies [chunk_f[c], chunk_f[c + 1]), at most
+  // kTc256ChunkKs (M = 256) or kTc512ChunkKs (M = 512) k-steps.
   int NCH;
   const int *chunk_f;     // [NCH + 1]
   // M = 256 kernel with the tcgen05 inverse DFT (null unless the handle uses
   // it; its k-steps are then ordered by contraction warp and parity): the
   // four BF16 DFT matrices Ee, Oe, Eo, Oo (64 angles x 64 frequencies,
   // canonical K-major core matrices).
-  // M = 512: the matrices Ee, Oe, Eo (128 x 128) and, per contraction warp,
-  // {its first k-step, its k-steps, k-steps of the even, of the odd slots (4 bits each)}.
-  const uint32_t *hyb_w;   // [kHyb256Mats * 2048] or [kHyb512Mats * 8192]
-  const int4 *hyb_sched;   // [16] (M = 512)
+  const uint32_t *hyb_w;   // [kHyb256Mats * 2048]
   int hyb_pattern;         // k-steps per slot: 0 = {3,2,2,2,1,1,1,1}, 1 = {3,3,2,2,2,2,2,2}
 };
 
 constexpr int kHyb256N0 = 3;    // k-steps of f = 0
 constexpr int kHyb256Mats = 4;
-constexpr int kHyb512Mats = 3;
 
 constexpr int kTc256ChunkKs = 22;
+constexpr int kTc512ChunkKs = 44;
+constexpr int kTc512MaxKsPerF = 6;  // rings with N_r <= 512 have r <= 81: at most 6 k-steps of 16 per frequency
 
 struct PolarArgs {
   const float *imgs;   // [n][L][L]
@@ -153,8 +152,6 @@ struct RescoreArgs {
 cudaError_t launch_refs16(const Geometry &g, const float2 *B, int ktiles, uint4 *B16, bool fp16, cudaStream_t st);
 // M = 256: mma.sync contraction with the tcgen05 inverse DFT.
 cudaError_t launch_cc_hybrid256(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st);
-// M = 512: the same.
-cudaError_t launch_cc_hybrid512(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st);
 cudaError_t launch_cc_tc(const Geometry &g, const TcArgs &a, bool fp16, cudaStream_t st);
 cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, unsigned long long *best,
                         cudaStream_t st);  // (clears best)
