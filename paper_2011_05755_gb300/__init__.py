@@ -341,7 +341,6 @@ class Aligner:
         self.L = L
         self.h = mra_create(L, first_ring, last_ring, ring_step, shift_range, shift_step, mirror, precision,
                             chunk_images, kernel)
-        self.K = 0
 
     def close(self):
         if getattr(self, "h", None) is not None and self.h.value:
@@ -358,14 +357,17 @@ class Aligner:
     def info(self) -> dict:
         return mra_get_info(self.h)
 
+    @property
+    def K(self) -> int:
+        """References the handle holds; calls on ``h`` itself (``mra_run_graph``, ``mra_run_host``) set them too."""
+        return self.info["K"] if self.h is not None else 0
+
     def set_refs(self, refs: torch.Tensor, stream=None):
         _check_stack(refs, self.L, "refs")
         mra_set_refs(self.h, refs, stream)
-        self.K = refs.shape[0]
 
     def copy_refs(self, other: "Aligner", stream=None):
         mra_copy_refs(self.h, other.h, stream)
-        self.K = other.K
 
     def align(self, imgs: torch.Tensor, poses=None, stream=None) -> torch.Tensor:
         _check_stack(imgs, self.L, "imgs")
@@ -376,16 +378,17 @@ class Aligner:
     def average(self, imgs, poses, avg=None, counts=None, stream=None):
         _check_stack(imgs, self.L, "imgs")
         _check_poses(poses, imgs.shape[0])
+        K = self.K
         if avg is not None:
             _check_stack(avg, self.L, "avg")
-            if avg.shape[0] != self.K:
-                raise ValueError(f"avg must hold K = {self.K} classes, got {avg.shape[0]}")
-        if counts is not None and tuple(counts.shape) != (self.K,):
-            raise ValueError(f"counts must have shape [{self.K}], got {list(counts.shape)}")
+            if avg.shape[0] != K:
+                raise ValueError(f"avg must hold K = {K} classes, got {avg.shape[0]}")
+        if counts is not None and tuple(counts.shape) != (K,):
+            raise ValueError(f"counts must have shape [{K}], got {list(counts.shape)}")
         if avg is None:
-            avg = torch.zeros((self.K, self.L, self.L), dtype=torch.float32, device=imgs.device)
+            avg = torch.zeros((K, self.L, self.L), dtype=torch.float32, device=imgs.device)
         if counts is None:
-            counts = torch.empty((self.K,), dtype=torch.int32, device=imgs.device)
+            counts = torch.empty((K,), dtype=torch.int32, device=imgs.device)
         mra_average(self.h, imgs, poses, avg, counts, stream)
         return avg, counts
 
@@ -404,5 +407,5 @@ class Aligner:
     def debug_cc(self, imgs, stream=None):
         _check_stack(imgs, self.L, "imgs")
         i = self.info
-        out = torch.empty((imgs.shape[0], self.K, i["S"], 2, i["M"]), dtype=torch.float32, device=imgs.device)
+        out = torch.empty((imgs.shape[0], i["K"], i["S"], 2, i["M"]), dtype=torch.float32, device=imgs.device)
         return mra_debug_cc(self.h, imgs, out, stream)
