@@ -227,7 +227,9 @@ int mra_run_host(mra_t h, const float *h_refs, int32_t K, const float *h_imgs, i
  * workspace); the second captures them into a graph (on a stream of the
  * handle; nothing runs during the capture) and launches it, and every
  * later call with the same buffers and sizes replays it.  A call with
- * other buffers or sizes drops the graph and starts again.  The buffers'
+ * other buffers or sizes drops the graph and starts again, and so does the
+ * first one after another call on the handle has reallocated one of its own
+ * buffers (references of another padded count, a larger n).  The buffers'
  * contents may change between calls; their addresses and sizes must not
  * while a graph is cached (the graph holds them, and the TMA descriptor of
  * the image stack).
@@ -236,7 +238,8 @@ int mra_run_host(mra_t h, const float *h_refs, int32_t K, const float *h_imgs, i
  * counterpart in the paper: this is launch plumbing. */
 int mra_run_graph(mra_t h, const float *d_refs, int32_t K, const float *d_imgs, int64_t n, mra_pose_t *d_poses,
                   float *d_avg, int32_t *d_counts, mra_stream_t stream);
-/* *captured = 1 once mra_run_graph holds an instantiated graph, else 0. */
+/* *captured = 1 while mra_run_graph holds an instantiated graph that its next
+ * call with the same buffers and sizes would replay, else 0. */
 int mra_graph_info(mra_t h, int32_t *captured);
 
 /* Wait for the handle's work on `stream`, then report device-side failures:

@@ -87,8 +87,13 @@ struct mra_handle {
     }
   };
   GraphKey graph_key{};
-  int graph_seen = 0;               // calls with graph_key so far (the graph is captured on the second)
+  bool graph_ready = false;         // the pass ran eagerly with graph_key: the next call captures it
   cudaGraphExec_t graph_exec = nullptr;
+  // A graph also holds addresses of the handle's own buffers (references,
+  // workspaces), which calls with another K or a larger n reallocate: it is
+  // valid while no buffer has been freed since the eager pass before it.
+  uint64_t frees = 0;               // device buffers freed so far (dev_free)
+  uint64_t graph_frees = 0;         // its value at that eager pass
   cudaStream_t capture_stream = nullptr;
   bool capturing = false;           // stage timing records are not taken inside a capture
   // per-stage event timing (mra_profile)
@@ -187,6 +192,7 @@ int dev_alloc(mra_handle *h, T **p, size_t bytes, const char *what) {
 
 void dev_free(mra_handle *h, void *p, size_t bytes) {
   if (p) {
+    ++h->frees;
     cudaFree(p);
     h->workspace -= (bytes == 0 ? 16 : bytes);
   }
@@ -1316,17 +1322,20 @@ int mra_run_graph(mra_t h, const float *d_refs, int32_t K, const float *d_imgs, 
     if (int rc = mra_align(h, d_imgs, n, d_poses, stream)) return rc;
     return mra_average(h, d_imgs, d_poses, n, d_avg, d_counts, stream);
   };
-  if (!(key == h->graph_key)) {  // new buffers or sizes: drop the old graph, run eagerly
+  if (!h->graph_ready || !(key == h->graph_key) || h->frees != h->graph_frees) {
+    // new buffers or sizes, the caller's or the handle's: drop the old graph and run eagerly, which sizes
+    // and allocates every workspace and sets every kernel attribute (neither may happen inside a capture)
     if (h->graph_exec) {
       cudaGraphExecDestroy(h->graph_exec);
       h->graph_exec = nullptr;
     }
+    h->graph_ready = false;
+    if (int rc = eager()) return rc;
     h->graph_key = key;
-    h->graph_seen = 0;
+    h->graph_frees = h->frees;
+    h->graph_ready = true;
+    return MRA_OK;
   }
-  // the first call with these buffers runs eagerly: it sizes and allocates every workspace and sets
-  // every kernel attribute, none of which may happen inside a capture
-  if (!h->graph_exec && h->graph_seen++ == 0) return eager();
   if (!h->graph_exec) {
     cudaError_t e;
     if (!h->capture_stream &&
@@ -1356,13 +1365,15 @@ int mra_run_graph(mra_t h, const float *d_refs, int32_t K, const float *d_imgs, 
     }
   }
   cudaError_t e = cudaGraphLaunch(h->graph_exec, st);
-  return e == cudaSuccess ? MRA_OK : cuda_err(h, e, "cudaGraphLaunch");
+  if (e != cudaSuccess) return cuda_err(h, e, "cudaGraphLaunch");
+  h->K = K;  // the pass sets the references; another call may have left fewer or more of the same padded count
+  return MRA_OK;
 }
 
 int mra_graph_info(mra_t h, int32_t *captured) {
   if (int rc = need_handle(h)) return rc;
   if (!captured) return set_err(h, MRA_EINVAL, "captured is NULL");
-  *captured = h->graph_exec ? 1 : 0;
+  *captured = h->graph_exec && h->frees == h->graph_frees ? 1 : 0;
   return MRA_OK;
 }
 
