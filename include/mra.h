@@ -70,8 +70,8 @@ enum mra_precision {
 };
 
 /* Tensor-core kernel of the 16-bit paths when M = 256 (rings up to 40); the
- * two compute the same table and differ only in speed.  Other M and the
- * FP32 path ignore the choice. */
+ * two compute the same table, up to its 16-bit rounding, at different speed.
+ * Other M and the FP32 path ignore the choice. */
 enum mra_kernel {
     MRA_KERNEL_AUTO = 0,     /* the library's default (the kernel of MRA_KERNEL_TCGEN05)       */
     MRA_KERNEL_MMA_SYNC = 1, /* warp-level mma.sync throughout                                 */
@@ -161,8 +161,9 @@ int mra_set_refs(mra_t h, const float *d_refs, int32_t K, mra_stream_t stream);
  * configuration, each with its own chunk workspace and stream, can align
  * against one reference set that was transformed once (Algorithm 1's
  * reference preparation is done per set, not per handle).  The two
- * configurations must agree in every field but chunk_images (else
- * MRA_EINVAL); src must hold references (else MRA_ESTATE).  The copy reads
+ * configurations must agree in every field but chunk_images and kernel (else
+ * MRA_EINVAL; between kernels that order the reference fragments differently
+ * the fragments are derived again from the spectra); src must hold references (else MRA_ESTATE).  The copy reads
  * src's buffers: the caller orders it after src's mra_set_refs (same stream,
  * or an event) and keeps src alive and its references unchanged until the
  * copy has run.  No paper counterpart: this is serving plumbing. */

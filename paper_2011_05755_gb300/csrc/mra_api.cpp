@@ -1094,12 +1094,11 @@ int mra_copy_refs(mra_t dst, mra_t src, mra_stream_t stream) {
   if (src == dst) return MRA_OK;
   if (src->K == 0) return set_err(dst, MRA_ESTATE, "source handle holds no references");
   const mra_config_t &a = dst->cfg, &b = src->cfg;
-  auto tcgen05 = [](mra_t h) { return h->half && h->g.M == 256 && h->cfg.kernel == MRA_KERNEL_TCGEN05; };
   if (a.L != b.L || a.first_ring != b.first_ring || a.last_ring != b.last_ring || a.ring_step != b.ring_step ||
       a.shift_range != b.shift_range || a.shift_step != b.shift_step || a.mirror != b.mirror ||
-      a.precision != b.precision || tcgen05(dst) != tcgen05(src))
+      a.precision != b.precision)
     return set_err(dst, MRA_EINVAL,
-                   "source and destination configurations differ (chunk_images may differ, the kernel may not)");
+                   "source and destination configurations differ (only chunk_images and the kernel may)");
   if (src->device != dst->device) return set_err(dst, MRA_EINVAL, "source handle lives on another device");
   if (int rc = select_device(dst)) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
