@@ -14,13 +14,16 @@ The library exposes two launch choices per handle (``mra_config_t``):
 :func:`tune` times every candidate on a synthetic stack of the
 configuration's shape (the alignment's work does not depend on the pixel
 values) with CUDA events and keeps the fastest.  Results are cached per
-(device, L, rings, shift grid, mirror, precision, K) in a JSON file
-(``MRA_TUNE_CACHE`` or ``~/.cache/mra_gb300/tune.json``), so a configuration
-is tuned once per machine.  :func:`tuned_aligner` builds an
+(device, L, rings, shift grid, mirror, precision, K) and library in a JSON
+file (``MRA_TUNE_CACHE`` or ``~/.cache/mra_gb300/tune.json``), so a
+configuration is tuned once per machine and version of the kernels: a choice
+measured with other kernels is not used (and replaced).  :func:`tuned_aligner` builds an
 :class:`~paper_2011_05755_gb300.Aligner` with the tuned choice.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
@@ -55,10 +58,26 @@ def candidates(first_ring: int, last_ring: int, ring_step: int, precision: int) 
     return [(k, c) for k in kernels for c in chunks]
 
 
+@functools.lru_cache(maxsize=None)
+def library_id() -> str:
+    """Identifies the kernels that a cached choice was measured with: a digest of the library's sources (or of
+    the library itself where it stands without them)."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    csrc, paths = os.path.join(here, "csrc"), []
+    if os.path.isdir(csrc):
+        paths = sorted(os.path.join(csrc, f) for f in os.listdir(csrc) if f.endswith((".cu", ".cuh", ".cpp", ".h")))
+    h = hashlib.sha256()
+    for p in paths or [os.path.join(here, "libmra.so")]:
+        h.update(os.path.basename(p).encode() + b"\0")
+        with open(p, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def _key(dev, L, first_ring, last_ring, ring_step, shift_range, shift_step, mirror, precision, K) -> str:
     name = torch.cuda.get_device_name(dev).replace(" ", "_")
     return (f"{name}|L{L}|r{first_ring}-{last_ring}-{ring_step}|s{shift_range:g}/{shift_step:g}|m{mirror}"
-            f"|p{precision}|K{K}")
+            f"|p{precision}|K{K}|lib{library_id()}")
 
 
 def _load(path: str) -> dict:
@@ -117,7 +136,8 @@ def tune(L: int, first_ring: int, last_ring: int, ring_step: int = 1, shift_rang
     best = min(results, key=lambda r: r["ms_per_image"])
     out = {"kernel": best["kernel"], "chunk_images": best["chunk_images"], "ms_per_image": best["ms_per_image"],
            "n_probe": n_probe, "candidates": results}
-    db = _load(path)
+    config = key.rsplit("|lib", 1)[0]  # this configuration's choices for other libraries go
+    db = {k: v for k, v in _load(path).items() if k.rsplit("|lib", 1)[0] != config}
     db[key] = out
     os.makedirs(os.path.dirname(path) or ".", exist_ok=True)
     tmp = path + ".tmp"
