@@ -246,7 +246,7 @@ template <int M, int KT, int RL>
 static cudaError_t launch_cc_t(const Geometry &g, const CCArgs &a, cudaStream_t st) {
   using Sh = CCShape<M, KT, RL>;
   const size_t smem = Sh::smem(a.seg_max);
-  static size_t granted = 0;
+  static SmemLimit granted;
   cudaError_t e = raise_smem_limit(cc_fp32_kernel<M, KT, RL>, smem, granted);
   if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + Sh::RT - 1) / Sh::RT;

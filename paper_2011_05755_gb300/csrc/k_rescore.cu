@@ -236,7 +236,7 @@ size_t rescore_smem(const Geometry &g) {
 // several geometries share the kernel).
 template <int M, bool PAIRS>
 static cudaError_t rescore_smem_attr(size_t smem) {
-  static size_t granted = 0;
+  static SmemLimit granted;
   return raise_smem_limit(rescore_kernel<M, PAIRS>, smem, granted);
 }
 
@@ -248,15 +248,10 @@ static cudaError_t launch_rescore_t(const Geometry &g, const RescoreArgs &a, cud
   // the image again, so only calls that leave SMs idle are split (top-8 and
   // rescore together: one image of 64 px 131 -> 27 us, 200 images of 76 px 241
   // -> 112 us, 107 with warp_fft_pairs).
-  static int at_once = 0;
-  if (at_once == 0) {
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    at_once = sms;
-  }
-  const int64_t slots = static_cast<int64_t>(at_once) * (2 * smem + 2048 > 233472 ? 1 : (4 * smem + 4096 > 233472 ? 2 : 4));
+  int sms = 0;
+  e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int64_t slots = static_cast<int64_t>(sms) * (2 * smem + 2048 > 233472 ? 1 : (4 * smem + 4096 > 233472 ? 2 : 4));
   unsigned parts = 1;
   while (parts < kTopRows && a.n * parts * 2 <= slots) parts *= 2;
   const dim3 grid(static_cast<unsigned>(a.n), parts);

@@ -920,7 +920,7 @@ template <int M, int KT, bool FP16>
 static cudaError_t launch_tc_t(const Geometry &g, const TcArgs &a, cudaStream_t st) {
   using Sh = TcShape<M, KT>;
   const size_t smem = Sh::smem(a.ks_max);
-  static size_t granted = 0;
+  static SmemLimit granted;
   cudaError_t e = raise_smem_limit(cc_tc_kernel<M, KT, FP16>, smem, granted);
   if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + Sh::RT - 1) / Sh::RT;
@@ -932,13 +932,9 @@ static cudaError_t launch_tc_t(const Geometry &g, const TcArgs &a, cudaStream_t 
 
 template <bool FP16>
 static cudaError_t launch_tc256(const Geometry &g, const TcArgs &a, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(cc_tc256_kernel<FP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kTc256Smem));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit granted;
+  const cudaError_t e = raise_smem_limit(cc_tc256_kernel<FP16>, kTc256Smem, granted);
+  if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
   if (row_tiles <= 0) return cudaSuccess;
   if (g.NCH > kTc256MaxChunks) return cudaErrorInvalidValue;
@@ -949,13 +945,9 @@ static cudaError_t launch_tc256(const Geometry &g, const TcArgs &a, cudaStream_t
 
 template <bool FP16>
 static cudaError_t launch_tc512(const Geometry &g, const TcArgs &a, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(cc_tc512_kernel<FP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kTc512Smem));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit granted;
+  const cudaError_t e = raise_smem_limit(cc_tc512_kernel<FP16>, kTc512Smem, granted);
+  if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
   if (row_tiles <= 0) return cudaSuccess;
   if (g.NCH > kTc512MaxChunks) return cudaErrorInvalidValue;

@@ -557,16 +557,15 @@ static int pick_splits(int64_t row_tiles, int ref_tiles, int sms) {
 
 template <int PATTERN, bool FP16>
 static cudaError_t launch_hybrid_t(const Geometry &g, const TcArgs &a, cudaStream_t st) {
-  static size_t granted = 0;
+  static SmemLimit granted;
   constexpr size_t smem = u256::z_stages(PATTERN) * u256::z_parities(PATTERN) * u256::kZStage + u256::kMisc +
                           (PATTERN == 0 ? 0 : HybPattern<PATTERN>::KS * 512);
   static_assert(smem <= kMaxSmemPerBlock, "row fragments must fit");
   if (g.KS != HybPattern<PATTERN>::KS) return cudaErrorInvalidValue;
   cudaError_t e = raise_smem_limit(cc_hybrid256_kernel<PATTERN, FP16>, smem, granted);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
   const int ref_tiles = (a.K + kTile - 1) / kTile;

@@ -381,21 +381,9 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   }
 }
 
-inline cudaError_t polar_sms(int *sms) {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
-  *sms = n;
-  return cudaSuccess;
-}
-
 template <int R, int MODE, int OUT>
 static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t smem, cudaStream_t st) {
-  static size_t granted = 0;
+  static SmemLimit granted;
   cudaError_t e = raise_smem_limit(polar_fft_kernel<R, MODE, OUT>, smem, granted);
   if (e != cudaSuccess) return e;
   // CTAs per image (each walks its share of the image's shift groups and
@@ -403,7 +391,7 @@ static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t 
   // stays small, one of those that fill an SM; more when the images are too
   // few for four waves.
   int sms = 0;
-  e = polar_sms(&sms);
+  e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   constexpr int kPerSm = 512 / polar_threads(MODE);
   const int64_t groups = (a.rows_per_img + R - 1) / R;
@@ -471,7 +459,7 @@ static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStr
   if (R > a.rows_per_img) R = a.rows_per_img;
   if constexpr (MODE != kPolarBare) {
     int sms = 0;
-    const cudaError_t e = polar_sms(&sms);
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     R = polar_bordered_rows(a, R, sms);
     const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
