@@ -269,19 +269,30 @@ size_t cc_fp32_smem(int M, int seg_max) {
   }
 }
 
+// M = 256: 8 x 8 tiles, one CTA of 16 warps per SM, or 8 x 4 tiles, two of 8
+// warps.  15.5 against 18.4 ms at K = 100 (13 and 25 tiles per row tile), 349
+// against 331 us at K = 10 (2 and 3), 1.98 against 1.33 ms at K = 1 (1 and 1): a
+// small tile costs 0.62 of a large one, so it can only win where it leaves out
+// enough padding references (K <= 4, 9..12).  A call of few tiles leaves SMs
+// idle either way and a pass of small tiles takes 1.23 times one of large ones
+// (half the warps for the frequencies of a tile; 76 px, K = 9: 63 row tiles 25.2
+// against 20.7 us, 125 row tiles 44.8 against 36.7, 188 row tiles 47.0 against 51.4).
+static bool small_tiles(const CCArgs &a) {
+  const int64_t row_tiles = (a.rows + kTile - 1) / kTile;
+  const int large = (a.K + 7) / 8, small = (a.K + 3) / 4;
+  int sms = 0;
+  if (0.62 * small >= large || sm_count(&sms) != cudaSuccess) return false;
+  const int64_t small_passes = (row_tiles * small + 2 * sms - 1) / (2 * sms), large_passes = (row_tiles * large + sms - 1) / sms;
+  return 1.23 * small_passes < large_passes;
+}
+
 cudaError_t launch_cc_fp32(const Geometry &g, const CCArgs &a, cudaStream_t st) {
   switch (g.M) {
     case 16: return launch_cc_t<16, 8, 2>(g, a, st);
     case 32: return launch_cc_t<32, 8, 2>(g, a, st);
     case 64: return launch_cc_t<64, 8, 2>(g, a, st);
     case 128: return launch_cc_t<128, 8, 2>(g, a, st);
-    case 256:
-      // 8 x 8 tiles, one CTA of 16 warps per SM, or 8 x 4 tiles, two of 8 warps:
-      // 15.5 against 18.4 ms at K = 100 (13 and 25 tiles per row tile), 349
-      // against 331 us at K = 10 (2 and 3), 1.98 against 1.33 ms at K = 1 (1 and
-      // 1): a small tile costs 0.62 of a large one, so it is taken where it
-      // leaves out enough padding references (K <= 4, 9..12)
-      return 0.62 * ((a.K + 3) / 4) < (a.K + 7) / 8 ? launch_cc_t<256, 4, 1>(g, a, st) : launch_cc_t<256, 8, 2>(g, a, st);
+    case 256: return small_tiles(a) ? launch_cc_t<256, 4, 1>(g, a, st) : launch_cc_t<256, 8, 2>(g, a, st);
     case 512: return launch_cc_t<512, 4, 2>(g, a, st);
     default: return cudaErrorInvalidValue;
   }
