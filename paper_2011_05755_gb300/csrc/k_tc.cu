@@ -906,6 +906,62 @@ __global__ void __launch_bounds__(kTopThreads) top8_kernel(const float *__restri
   }
 }
 
+// The same by one warp per image: each lane keeps the eight largest of its
+// rows in order, the warp merges them.  Faster where an image has few rows or
+// the images are many (launch_top8).
+__global__ void __launch_bounds__(kTopThreads) top8_warp_kernel(const float *__restrict__ rowmax, int64_t n, int nrows,
+                                                                int *cand, unsigned long long *best_key) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t img = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
+  if (img >= n) return;
+  if (lane == 0) best_key[img] = 0ull;
+  float v[kTopRows];
+  int id[kTopRows];
+#pragma unroll
+  for (int e = 0; e < kTopRows; ++e) {
+    v[e] = -INFINITY;
+    id[e] = 0x7fffffff;
+  }
+  const float *rm = rowmax + img * nrows;
+  for (int j = lane; j < nrows; j += 32) {
+    const float x = rm[j];
+    if (x > v[kTopRows - 1]) {
+      v[kTopRows - 1] = x;
+      id[kTopRows - 1] = j;
+#pragma unroll
+      for (int e = kTopRows - 1; e > 0; --e)
+        if (v[e] > v[e - 1]) {
+          const float tv = v[e];
+          v[e] = v[e - 1];
+          v[e - 1] = tv;
+          const int ti = id[e];
+          id[e] = id[e - 1];
+          id[e - 1] = ti;
+        }
+    }
+  }
+  for (int round = 0; round < kTopRows; ++round) {
+    unsigned long long key = (v[0] == -INFINITY) ? 0ull : make_key(v[0], static_cast<uint32_t>(id[0]));
+    unsigned long long best = key;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
+      best = o > best ? o : best;
+    }
+    if (lane == 0) cand[img * kTopRows + round] = best ? static_cast<int>(0xffffffffu - static_cast<uint32_t>(best)) : -1;
+    const unsigned win = __ballot_sync(0xffffffffu, best != 0 && key == best);
+    if (best != 0 && lane == __ffs(win) - 1) {
+#pragma unroll
+      for (int e = 0; e < kTopRows - 1; ++e) {
+        v[e] = v[e + 1];
+        id[e] = id[e + 1];
+      }
+      v[kTopRows - 1] = -INFINITY;
+      id[kTopRows - 1] = 0x7fffffff;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // launchers (the FP32 rescore kernel is in k_rescore.cu)
 // ---------------------------------------------------------------------------
@@ -974,7 +1030,20 @@ cudaError_t launch_cc_tc(const Geometry &g, const TcArgs &a, bool fp16, cudaStre
 cudaError_t launch_top8(const float *rowmax, int64_t n, int nrows, int *cand, unsigned long long *best,
                         cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  top8_kernel<<<static_cast<unsigned>(n), kTopThreads, 0, st>>>(rowmax, nrows, cand, best);
+  // A CTA has a fixed cost of some 6 us and eight run on an SM, a warp's chain
+  // grows with the rows (us by warp / by CTA; rows: 150 images, 1,200, 20,000):
+  //     150: 6.2 / 6.5, 6.4 / 10.5, 21 / 92      600: 8.5 / 7.5,  8.6 / 10.5, 43 / 97
+  //     300: 6.4 / 6.5, 6.5 / 10.5, 29 / 93    1,200: 12.5 / 8.3, 12.5 / 10.8, 82 / 109
+  //                                            2,400: 20.6 / 8.4, 20.6 / 12.5, 148 / 133
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  if (nrows <= 300 || (nrows <= 1200 && n > 8 * static_cast<int64_t>(sms))) {
+    constexpr int kWarps = kTopThreads / 32;
+    top8_warp_kernel<<<static_cast<unsigned>((n + kWarps - 1) / kWarps), kTopThreads, 0, st>>>(rowmax, n, nrows, cand, best);
+  } else {
+    top8_kernel<<<static_cast<unsigned>(n), kTopThreads, 0, st>>>(rowmax, nrows, cand, best);
+  }
   return cudaGetLastError();
 }
 
