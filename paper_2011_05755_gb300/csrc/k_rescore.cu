@@ -23,8 +23,8 @@ constexpr int kRescoreThreads = 256;  // 8 warps per CTA (one image)
 // Registers are held to 64 per thread for M = 32..256, so that four CTAs
 // (images) fit on an SM where their shared memory allows (the 76-pixel
 // workload).
-// PAIRS: ring transforms by warp_fft_pairs (M >= 256, and more candidates
-// than one to a CTA).
+// PAIRS: ring transforms by warp_fft_pairs (M >= 256, enough long rings, and
+// more candidates than one to a CTA).
 template <int M, bool PAIRS>
 __global__ void __launch_bounds__(kRescoreThreads, (M >= 32 && M <= 256) ? 4 : 1)
     rescore_kernel(Geometry g, RescoreArgs a) {
@@ -255,7 +255,13 @@ static cudaError_t launch_rescore_t(const Geometry &g, const RescoreArgs &a, cud
   unsigned parts = 1;
   while (parts < kTopRows && a.n * parts * 2 <= slots) parts *= 2;
   const dim3 grid(static_cast<unsigned>(a.n), parts);
-  if (M >= 256 && parts < kTopRows) {
+  // Two-stage ring transforms: where enough rings are long.  M = 256, by the
+  // rings of 256 samples among 1..r, plain / pairs (us, 300 and 5,000 images of
+  // 84 px): 1 (r = 21) 68 / 72 and 902 / 912; 4 (24) 79 / 81 and 1,056 / 1,028;
+  // 6 (26) 88 / 89 and 1,207 / 1,144; 8 (28) 99 / 97 and 1,396 / 1,300;
+  // 20 (40) 193 / 179 and 2,421 / 2,127; M = 512 gains 8 to 15 % throughout.
+  const bool long_rings = M >= 512 || (M == 256 && g.cls[1].i1 - g.cls[1].i0 >= 6);
+  if (M >= 256 && long_rings && parts < kTopRows) {
     e = rescore_smem_attr<M, (M >= 256)>(smem);
     if (e != cudaSuccess) return e;
     rescore_kernel<M, (M >= 256)><<<grid, kRescoreThreads, smem, st>>>(g, a);

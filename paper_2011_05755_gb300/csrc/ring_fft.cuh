@@ -88,10 +88,11 @@ __device__ __forceinline__ void warp_fft_inplace(float2 *z, int H, int logH, int
 // transform but leaves most lanes idle on rings of 64 samples and fewer: the
 // rescore of 12,000 images of 76 px (M = 256) takes 5.06 -> 4.60 ms, of 600
 // images of 128 px (M = 512) 1.72 -> 1.51 ms, of 5,003 images of 32 px
-// (M = 128) 0.44 -> 0.52 ms, hence M >= 256 only.  Where each candidate has a
-// CTA of its own (a few images), the shorter chain of the plain transform is
-// faster instead (one image of 64 px: 46 against 49 us for the whole call).  Not inlined: inlined, its
-// addresses are kept across the candidates and spill (4.71 ms).
+// (M = 128) 0.44 -> 0.52 ms, hence M >= 256 with enough rings of 256 samples
+// only.  Where each candidate has a CTA of its own (a few images), the shorter
+// chain of the plain transform is faster instead (one image of 64 px: 46 against
+// 49 us for the whole call).  Not inlined: inlined, its addresses are kept across
+// the candidates and spill (4.71 ms).
 __device__ __forceinline__ int fft_swz(int i) { return i ^ (((i >> 4) & 3) << 2); }
 
 __device__ __forceinline__ void butterfly(float2 &u, float2 &v, float2 w) {
