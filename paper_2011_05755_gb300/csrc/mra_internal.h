@@ -164,6 +164,7 @@ size_t polar_smem_one_row(const Geometry &g, int mode, bool out16);
 int polar_rows_per_cta(const Geometry &g, int mode, bool out16);
 size_t cc_fp32_smem(int M, int seg_max);
 constexpr size_t kMaxSmemPerBlock = 232448;  // 227 KB
+constexpr size_t kSmemPerSm = 233472;        // 228 KB, of which each resident CTA takes 1 KB more than it asks for
 // Every check mra_create makes on a configuration, without CUDA calls or heap
 // use: MRA_OK, MRA_EINVAL or MRA_EUNSUPPORTED with a message in why.
 int check_config(const mra_config_t *c, char *why, size_t why_len);

@@ -128,7 +128,8 @@ __host__ __device__ inline int image_floats(const Geometry &g, int mode) {
 }
 
 // Threads of a CTA: with a bordered image one CTA of 16 warps fills an SM and
-// takes as many rows as fit (launch_polar_t); otherwise two of 8 warps.
+// takes as many rows as fit, unless the box is small or the image has one row
+// (launch_polar_t); otherwise two of 8 warps.
 __host__ __device__ constexpr int polar_threads(int mode) { return mode != kPolarBare ? 512 : 256; }
 
 // Bilinear interpolation with the fused multiply-adds written out: left to
@@ -139,10 +140,9 @@ __device__ __forceinline__ float bilerp(float fx, float fy, float gx, float gy, 
   return fmaf(gy, t, __fmul_rn(fy, b));
 }
 
-template <int R, int MODE, int OUT>
-__global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
+template <int R, int MODE, int OUT, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) polar_fft_kernel(Geometry g, const __grid_constant__ PolarArgs a) {
   extern __shared__ float4 smem_f4[];
-  constexpr int NT = polar_threads(MODE);
   const int L = g.L, NS = g.NS, M = g.M;
   const int NSp = sample_stride(g.NSb);
   const int LL = L * L;
@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
     int fw = 0;  // warp that takes the first pass of the next class
     sfor<0, kRingClasses>([&](auto kk) {  // longest first; a class the geometry lacks has no jobs
       constexpr int k = decltype(kk)::value;
-      fw = ring_class<(256 >> k), R, OUT, polar_threads(MODE) / 32>(g, a, smem, planes, NB16, tws, s_kpos, g.cls[k],
-                                                                    nrows, row0, warp, lane, fw);
+      fw = ring_class<(256 >> k), R, OUT, NT / 32>(g, a, smem, planes, NB16, tws, s_kpos, g.cls[k], nrows, row0, warp,
+                                                   lane, fw);
     });
 
     if constexpr (MODE == kPolarInt) load_taps(threadIdx.x);
@@ -381,10 +381,10 @@ __global__ void __launch_bounds__(polar_threads(MODE), 512 / polar_threads(MODE)
   }
 }
 
-template <int R, int MODE, int OUT>
+template <int R, int MODE, int OUT, int NT = polar_threads(MODE)>
 static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t smem, cudaStream_t st) {
   static SmemLimit granted;
-  cudaError_t e = raise_smem_limit(polar_fft_kernel<R, MODE, OUT>, smem, granted);
+  cudaError_t e = raise_smem_limit(polar_fft_kernel<R, MODE, OUT, NT>, smem, granted);
   if (e != cudaSuccess) return e;
   // CTAs per image (each walks its share of the image's shift groups and
   // stages the image once): four of the small CTAs, so that the last wave
@@ -393,14 +393,14 @@ static cudaError_t launch_polar_r(const Geometry &g, const PolarArgs &a, size_t 
   int sms = 0;
   e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  constexpr int kPerSm = 512 / polar_threads(MODE);
+  constexpr int kPerSm = 512 / NT;
   const int64_t groups = (a.rows_per_img + R - 1) / R;
   const int64_t want = (static_cast<int64_t>(4 * kPerSm) * sms + a.n_imgs - 1) / a.n_imgs;
   int64_t per_img = kPerSm > 1 && smem + 1024 <= 232448 / 2 ? 4 : 1;
   if (per_img < want) per_img = want;
   if (per_img > groups) per_img = groups;
   dim3 grid(static_cast<unsigned>(per_img), static_cast<unsigned>(a.n_imgs));
-  polar_fft_kernel<R, MODE, OUT><<<grid, polar_threads(MODE), smem, st>>>(g, a);
+  polar_fft_kernel<R, MODE, OUT, NT><<<grid, NT, smem, st>>>(g, a);
   return cudaGetLastError();
 }
 
@@ -461,6 +461,25 @@ static cudaError_t launch_polar_t(const Geometry &g, const PolarArgs &a, cudaStr
     int sms = 0;
     const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
+    // CTAs of 8 warps, two per SM, where one of 16 leaves its warps or the SM
+    // idle (us, 16 warps / 8):
+    // * one row per image (no shifts, or references), nothing for the other
+    //   CTA's latency to hide behind: 300 images of 12, 60, 76 px 14.3 / 10.1,
+    //   20.9 / 14.1, 22.4 / 15.0; 8,000 of 12, 76 px 194 / 98, 359 / 259 (and
+    //   128 px, where only one CTA fits either way, 207 / 228: not taken);
+    // * boxes whose rings hold fewer samples than the large CTA has threads
+    //   (last ring up to 10), 4 rows a CTA: 2,000 images of 12, 24 px with 25
+    //   shifts 228 / 168, 317 / 276;
+    // * up to twice that where the images are so few that each is staged by
+    //   several CTAs, or have 4 rows: 300 images of 32 px, 25 shifts 79 / 64, but
+    //   2,000 392 / 460; 2,000 with 4 shifts 82 / 53.
+    const size_t smem1 = polar_smem_bytes(g, MODE, OUT != kOutF32, 1);
+    if (a.rows_per_img == 1 && 2 * (smem1 + 1024) <= kSmemPerSm)
+      return launch_polar_r<1, MODE, OUT, 256>(g, a, smem1, st);
+    const size_t smem4 = polar_smem_bytes(g, MODE, OUT != kOutF32, 4);
+    if (R >= 4 && 2 * (smem4 + 1024) <= kSmemPerSm &&
+        (g.NS < 512 || (g.NS < 1024 && (a.n_imgs < 4 * static_cast<int64_t>(sms) || a.rows_per_img == 4))))
+      return launch_polar_r<4, MODE, OUT, 256>(g, a, smem4, st);
     R = polar_bordered_rows(a, R, sms);
     const size_t smem = polar_smem_bytes(g, MODE, OUT != kOutF32, R);
     switch (R) {
