@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -204,17 +205,36 @@ int check_launch(mra_handle *h, cudaError_t e, const char *what) {
   return MRA_OK;
 }
 
-template <class T>
-int upload(mra_handle *h, const std::vector<T> &v, const T **out, const char *what) {
-  T *d = nullptr;
-  int rc = dev_alloc(h, &d, v.size() * sizeof(T), what);
-  if (rc) return rc;
-  h->tables.push_back(d);
-  cudaError_t e = cudaMemcpy(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_err(h, e, what);
-  *out = d;
-  return MRA_OK;
-}
+// The geometry tables of a handle: collected on the host, put into one device
+// buffer by one copy, and each table's address set then (seventeen allocations
+// and copies took a good part of mra_create).
+class TableSet {
+ public:
+  template <class T>
+  void add(const std::vector<T> &v, const T **out) {
+    const size_t at = (bytes_.size() + 255) & ~size_t(255);
+    bytes_.resize(at + v.size() * sizeof(T));
+    std::memcpy(bytes_.data() + at, v.data(), v.size() * sizeof(T));
+    slots_.push_back({at, [out](const unsigned char *d) { *out = reinterpret_cast<const T *>(d); }});
+  }
+  int upload(mra_handle *h) const {
+    unsigned char *d = nullptr;
+    if (int rc = dev_alloc(h, &d, bytes_.size(), "geometry tables")) return rc;
+    h->tables.push_back(d);
+    const cudaError_t e = cudaMemcpy(d, bytes_.data(), bytes_.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return cuda_err(h, e, "copy geometry tables");
+    for (const Slot &slot : slots_) slot.set(d + slot.at);
+    return MRA_OK;
+  }
+
+ private:
+  struct Slot {
+    size_t at;
+    std::function<void(const unsigned char *)> set;
+  };
+  std::vector<unsigned char> bytes_;
+  std::vector<Slot> slots_;
+};
 
 }  // namespace
 
@@ -464,7 +484,6 @@ int build_tables(mra_handle *h) {
       ksinfo = info;
     }
   }
-  std::vector<int> binpos16(NBIN);
   std::vector<int> binpos(NBIN);
   std::vector<float> bweight(NBIN);
   std::vector<float2> offs(NS);
@@ -472,7 +491,6 @@ int build_tables(mra_handle *h) {
     const int N = NN[i];
     for (int f = 0; f <= N / 2; ++f) {
       binpos[rings[i].z + f] = fseg[f].x + (i - first[f]);
-      binpos16[rings[i].z + f] = kso[f] * 16 + (i - first[f]);
       double w = kTwoPi * rr[i] * c.ring_step / (double(N) * double(N));
       if (f == N / 2 && N < M) w *= 0.5;  // Nyquist split of an inner ring
       bweight[rings[i].z + f] = static_cast<float>(w);
@@ -513,17 +531,17 @@ int build_tables(mra_handle *h) {
   g.mirror = c.mirror;
   h->NBIN = NBIN;
   h->NB = NB;
-  int rc;
-  if ((rc = upload(h, offs, &g.offs, "ring offsets"))) return rc;
+  TableSet tables;
+  tables.add(offs, &g.offs);
   g.taps = nullptr;
-  if ((rc = upload(h, rings, &g.rings, "ring table"))) return rc;
-  if ((rc = upload(h, binpos, &g.binpos, "bin positions"))) return rc;
-  if ((rc = upload(h, bweight, &g.bweight, "ring weights"))) return rc;
-  if ((rc = upload(h, fwd, &g.fwd_tw, "forward twiddles"))) return rc;
-  if ((rc = upload(h, inv, &g.inv_tw, "inverse twiddles"))) return rc;
-  if ((rc = upload(h, shifts, &g.shifts, "shift grid"))) return rc;
-  if ((rc = upload(h, ang, &g.angles, "angle table"))) return rc;
-  if ((rc = upload(h, fseg, &g.fseg, "frequency segments"))) return rc;
+  tables.add(rings, &g.rings);
+  tables.add(binpos, &g.binpos);
+  tables.add(bweight, &g.bweight);
+  tables.add(fwd, &g.fwd_tw);
+  tables.add(inv, &g.inv_tw);
+  tables.add(shifts, &g.shifts);
+  tables.add(ang, &g.angles);
+  tables.add(fseg, &g.fseg);
   g.KS = static_cast<int>(ksinfo.size());
   // Polar kernel: the image inside a zero border that every neighbour of every
   // sample stays in, where the border needs at most 8 pixels (the sample
@@ -578,33 +596,36 @@ int build_tables(mra_handle *h) {
     mra::set_ring_classes(g, rings.data(), NR, gap);
     if (g.mode != mra::kPolarBare) {
       // samples in patches of up to 5 rings of one length x 8 angles
-      std::vector<float4> taps;
-      taps.reserve(NS);
+      std::vector<float4> taps(NS);
+      float4 *tap = taps.data();
       for (int i0 = 0, i1; i0 < NR; i0 = i1) {
         for (i1 = i0 + 1; i1 < NR && i1 < i0 + 5 && NN[i1] == NN[i0];) ++i1;
-        for (int q0 = 0; q0 < NN[i0]; q0 += 8)
+        for (int q0 = 0; q0 < NN[i0]; q0 += 8)  // (every ring has a multiple of 8 samples)
           for (int i = i0; i < i1; ++i)
-            for (int k = q0; k < q0 + 8 && k < NN[i]; ++k) {
+            for (int k = q0; k < q0 + 8; ++k) {
               const int q = rings[i].y + k, at = (rings[i].y + gap * i + k) | q << 16;
               float fat, fidx;
               std::memcpy(&fat, &at, 4);
               if (g.mode == mra::kPolarFrac) {
-                taps.push_back(make_float4(fat, offs[q].x, offs[q].y, 0.f));
+                *tap++ = make_float4(fat, offs[q].x, offs[q].y, 0.f);
                 continue;
               }
               const float x = c0 + offs[q].x, y = c0 + offs[q].y;
-              const float xf = std::floor(x), yf = std::floor(y);
-              const int idx = (static_cast<int>(yf) + g.pad) * g.pitch + static_cast<int>(xf) + g.pad;
+              int xi = static_cast<int>(x), yi = static_cast<int>(y);  // floor
+              xi -= static_cast<float>(xi) > x;
+              yi -= static_cast<float>(yi) > y;
+              const int idx = (yi + g.pad) * g.pitch + xi + g.pad;
               std::memcpy(&fidx, &idx, 4);
-              taps.push_back(make_float4(fidx, x - xf, y - yf, fat));
+              *tap++ = make_float4(fidx, x - static_cast<float>(xi), y - static_cast<float>(yi), fat);
             }
       }
-      if ((rc = upload(h, taps, &g.taps, "sample table"))) return rc;
+      tables.add(taps, &g.taps);
     }
   }
-  if ((rc = upload(h, kso, &g.kso, "k-step offsets"))) return rc;
-  if ((rc = upload(h, ksinfo, &g.ksinfo, "k-step table"))) return rc;
-  if ((rc = upload(h, binpos16, &g.binpos16, "16-bit bin positions"))) return rc;
+  if (h->half) {
+    tables.add(kso, &g.kso);
+    tables.add(ksinfo, &g.ksinfo);
+  }
   {
     // per-frequency bases: position of (ring i, f) = base[f] + i in both layouts
     std::vector<int> kpos(H + 1), kpos16(H + 1);
@@ -612,8 +633,8 @@ int build_tables(mra_handle *h) {
       kpos[f] = fseg[f].x - first[f];
       kpos16[f] = kso[f] * 16 - first[f];
     }
-    if ((rc = upload(h, kpos, &g.kpos, "frequency bases"))) return rc;
-    if ((rc = upload(h, kpos16, &g.kpos16, "16-bit frequency bases"))) return rc;
+    tables.add(kpos, &g.kpos);
+    if (h->half) tables.add(kpos16, &g.kpos16);
   }
   if (h->half && pattern < 0 && M >= 256) {
     // whole frequencies per staging chunk of the MRA_KERNEL_MMA_SYNC (M = 256) and M = 512 kernels, greedily
@@ -627,13 +648,13 @@ int build_tables(mra_handle *h) {
     }
     chunk_f.push_back(H + 1);
     g.NCH = static_cast<int>(chunk_f.size()) - 1;
-    if ((rc = upload(h, chunk_f, &g.chunk_f, "staging chunks"))) return rc;
+    tables.add(chunk_f, &g.chunk_f);
   }
-  // BF16 fragments of the 16-point DFT matrices for the tensor-core inverse DFT.
+  // BF16 fragments of the 16-point DFT matrices for the mma.sync inverse DFT.
   // Stage 1 (A, rows (re/im, k), cols (re/im, a)): [[C, -S], [S, C]];
   // stage 2 (B, rows (re/im, t), cols (re/im, j)): [[C, S], [-S, C]];
   // C = cos(2 pi x y / 16), S = sin(2 pi x y / 16).  Lane 4g + t4 of a warp.
-  {
+  if (h->half && pattern < 0 && M >= 256) {
     std::vector<uint32_t> frag(1024);
     auto h16 = [](double v) { return static_cast<uint32_t>(bf16_bits(v)); };
     auto F = [](int blk_r, int blk_c, int x, int y, bool stage2) {
@@ -666,13 +687,14 @@ int build_tables(mra_handle *h) {
           }
         }
     }
-    if ((rc = upload(h, frag, &g.dft16, "DFT fragments"))) return rc;
+    tables.add(frag, &g.dft16);
   }
   if (pattern >= 0) {
-    if ((rc = upload(h, hybrid_matrices(), &g.hyb_w, "inverse-DFT matrices"))) return rc;
+    tables.add(hybrid_matrices(), &g.hyb_w);
     g.hyb_pattern = pattern;
   }
-  if ((rc = dev_alloc(h, &h->d_err, sizeof(int), "failure flags"))) return rc;
+  if (int rc = tables.upload(h)) return rc;
+  if (int rc = dev_alloc(h, &h->d_err, sizeof(int), "failure flags")) return rc;
   h->tables.push_back(h->d_err);
   cudaError_t e = cudaMemset(h->d_err, 0, sizeof(int));
   if (e != cudaSuccess) return cuda_err(h, e, "cudaMemset(failure flags)");
