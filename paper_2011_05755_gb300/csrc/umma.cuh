@@ -1,7 +1,7 @@
 // Blackwell (sm_103a) tensor-core primitives written as inline PTX: tensor
-// memory (TMEM) allocation, loads and stores, the 5th-generation MMA
-// (tcgen05.mma, BF16/FP16 operands, FP32 accumulation in TMEM), its commit
-// to an mbarrier, shared-memory matrix descriptors, and TMA tensor-map loads.
+// memory (TMEM) allocation and loads, the 5th-generation MMA (tcgen05.mma,
+// BF16/FP16 operands, FP32 accumulation in TMEM), its commit to an mbarrier,
+// shared-memory matrix descriptors, and waits that give up with the CTA.
 //
 // Operand layout used throughout (the "K-major, no swizzle" canonical
 // layout): a matrix of R rows by 16 K-elements (16-bit) is stored as core
@@ -72,11 +72,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Hint to bring `bytes` (a multiple of 16) of global memory at `src` into L2.
-__device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
 
 // Non-blocking test of an mbarrier phase.
 __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
