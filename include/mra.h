@@ -71,7 +71,9 @@ enum mra_precision {
 
 /* Tensor-core kernel of the 16-bit paths when M = 256 (rings up to 40); the
  * two compute the same table, up to its 16-bit rounding, at different speed.
- * Other M and the FP32 path ignore the choice. */
+ * (The table picks the rows that are rescored in FP32, so an image whose best
+ * rows are nearly tied can get another of them as its pose.)  Other M and the
+ * FP32 path ignore the choice. */
 enum mra_kernel {
     MRA_KERNEL_AUTO = 0,     /* the library's default (the kernel of MRA_KERNEL_TCGEN05)       */
     MRA_KERNEL_MMA_SYNC = 1, /* warp-level mma.sync throughout                                 */
